@@ -8,9 +8,14 @@
 //      keep the n rows that land on I;
 //   3. row pass: inverse FFT along x2, keep the n columns on I, fused epilogue
 //      (u + ., u + m.*., or -.).
-// The FFT is a shared-memory Stockham autosort transform with radix-4 stages
-// (one radix-2 stage when log2 L is odd).
+// For line lengths 64 .. 2048 (n from 17 to 1024) the three passes run in
+// 64-bit fixed point (fx_line.cuh, fx_fft.cu).  The FP64 kernels below, a
+// shared-memory Stockham autosort transform with radix-4 stages (one radix-2
+// stage when log2 L is odd), keep the other lengths (below 64 there is too
+// little to gain; 4096 would need a plan with more passes to keep the
+// fixed-point error below that of FP64) and build the kernel transform.
 #include "fft_line.cuh"
+#include "fx_fft.cuh"
 #include "lss_common.cuh"
 #include "lss_ctx.h"
 #include "lss3d.h"
@@ -126,11 +131,71 @@ constexpr int kFftSmax = 200 * 1024;   // dynamic shared memory the FFT kernels 
 
 int col_group(const lss_ctx* c) { return c->tune.fft_C ? c->tune.fft_C : col_group(c->L); }
 
+// The three passes in fixed point: rows -> transformed rows, columns in place
+// through the kernel transform, rows back with the epilogue.  Scratch: the
+// n x L entries per right-hand side, an exponent per row and per column, and
+// for plane waves exp(i omega d_a p) along each axis.
+int matvec_fx(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int out_mode, const double* dirs_dev,
+              double2* uI, cudaStream_t s) {
+    const int n = c->n, L = c->L, lg = c->lgL;
+    const long long ent = (long long)n * L;
+    const size_t buf = (size_t)ent * R * sizeof(longlong2), pha = (size_t)R * 2 * n * sizeof(double2);
+    int rc = lss_grow(c, (void**)&c->mv_buf, &c->mv_cap, buf + pha + (size_t)(n + L) * R * sizeof(int));
+    if (rc) return rc;
+    double2* phase = (double2*)((char*)c->mv_buf + buf);
+    int* e1 = (int*)((char*)phase + pha);
+    int* e2 = e1 + (long long)n * R;
+    const bool pw = in_mode == MV_IN_PLANEWAVE;
+    const int E = lss_fx_entries(lg, (long long)L * L * R, c->num_sms);
+    ProfScope ps(c, s, LSS_PROF_MATVEC, pw ? 4 : 3);
+    FxArgs A{};
+    A.n = n;
+    A.dim = 2;
+    A.N = (long long)n * n;
+    A.tw = c->fx_tw;
+    A.khat = (const fx_tw*)c->fx_khat;
+    A.ek = c->fx_ek;
+    A.x = x;
+    A.m = c->m;
+    A.y = y;
+    A.uI = uI;
+    A.phase = phase;
+    A.in_mode = in_mode;
+    A.out_mode = out_mode;
+    A.in = A.out = (longlong2*)c->mv_buf;
+    A.in_r = A.out_r = ent;
+    cudaError_t e = cudaSuccess;
+    if (pw) e = lss_fx_phases(dirs_dev, phase, 2, n, R, c->omega, c->h, s);
+    // rows: line = row
+    A.nlines = A.lb = n;
+    A.out_b = A.in_b = L;
+    A.out_s = A.in_s = 1;
+    A.eout = e1;
+    if (!e) e = lss_fx_pass(FX_FWD_IN, lg, E, A, R, s);
+    // columns: line = storage position along a row, entry = row
+    A.nlines = A.lb = L;
+    A.out_b = A.in_b = 1;
+    A.out_s = A.in_s = L;
+    A.ein = e1;
+    A.ein_r = n;
+    A.ein_s = 1;
+    A.eout = e2;
+    if (!e) e = lss_fx_pass(FX_CONV, lg, E, A, R, s);
+    A.nlines = A.lb = n;
+    A.in_b = L;
+    A.in_s = 1;
+    A.ein = e2;
+    A.ein_r = L;
+    if (!e) e = lss_fx_pass(FX_INV_OUT, lg, E, A, R, s);
+    return lss_check_cuda(c, e, "fixed-point matvec launch");
+}
+
 }  // namespace
 
 std::vector<int> lss_fft_col_candidates(const lss_ctx* c) {
     std::vector<int> out;
     const int L = c->L;
+    if (lss_fx_supported(c->lgL)) return {lss_fx_lines(c->lgL)};
     for (int C : {1, 2, 4, 8})
         if (L % C == 0 && C * line_threads(L) <= 1024 && 2 * (size_t)C * L * sizeof(double2) <= (size_t)kFftSmax)
             out.push_back(C);
@@ -141,6 +206,7 @@ int lss_matvec(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int
                const double* dirs_dev, double2* uI, cudaStream_t s) {
     if (c->dim == 3) return lss3_matvec(c, x, y, R, in_mode, out_mode, dirs_dev, uI, s);
     const int n = c->n, L = c->L, lg = c->lgL;
+    if (lss_fx_supported(lg)) return matvec_fx(c, x, y, R, in_mode, out_mode, dirs_dev, uI, s);
     const size_t need = (size_t)n * L * R * sizeof(double2);
     int rc = lss_grow(c, (void**)&c->mv_buf, &c->mv_cap, need);
     if (rc) return rc;
@@ -195,7 +261,15 @@ int lss_fft_kernel_table(lss_ctx* c, const double2* kc, cudaStream_t s) {
     const double scale = c->omega * c->omega / ((double)L * (double)L);
     mv_cols<false><<<dim3(L / C, 1), C * nt, 2 * (size_t)C * L * sizeof(double2), s>>>(
         c->mv_buf, nullptr, c->khatT, c->tw, L, L, lg, C, scale);
-    return lss_check_cuda(c, cudaGetLastError(), "kernel table fft");
+    rc = lss_check_cuda(c, cudaGetLastError(), "kernel table fft");
+    if (!rc && lss_fx_supported(lg)) {
+        rc = lss_fx_tables(c, c->khatT, s);
+        if (!rc) {
+            cudaFree(c->khatT);
+            c->khatT = nullptr;
+        }
+    }
+    return rc;
 }
 
 // Opt the FFT kernels into large dynamic shared memory once per device.

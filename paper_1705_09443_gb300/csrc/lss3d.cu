@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "fft_line.cuh"
+#include "fx_fft.cuh"
 #include "lss_common.cuh"
 #include "lss_ctx.h"
 #include "lss3d.h"
@@ -1144,6 +1145,13 @@ int build_kernel3(lss_ctx* c, cudaStream_t s) {
     cudaFree(kc);
     cudaFree(tmp);
     if (!rc) rc = lss_check_cuda(c, e, "3D kernel table");
+    if (!rc && lss_fx_supported(lg)) {
+        rc = lss_fx_tables(c, d->khat, s);
+        if (!rc) {
+            cudaFree(d->khat);
+            d->khat = nullptr;
+        }
+    }
     return rc;
 }
 
@@ -1638,10 +1646,121 @@ int lss3_slab_apply(lss_ctx* c, int slab, const double2* v, double2* w, int R, c
     return sweep3_t<float2>(c, nullptr, w, R, slab, v, s);
 }
 
+// The operator in 64-bit fixed point (fx_line.cuh): x3 lines, x2 lines, x1
+// lines through the kernel transform, and back.
+static int matvec3_fx(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int out_mode,
+                      const double* dirs_dev, double2* uI, cudaStream_t s) {
+    Ctx3* d = c->d3;
+    const long long n = c->n, L = c->L;
+    const int lg = c->lgL;
+    const size_t ba = (size_t)n * n * L * R * sizeof(longlong2), pha = (size_t)R * 3 * n * sizeof(double2);
+    const size_t ne = (size_t)R * (n * n + 2 * n * L + L * L);
+    int rc = lss_grow(c, (void**)&d->mvA, &d->mvA_cap, ba + pha + ne * sizeof(int));
+    if (!rc) rc = lss_grow(c, (void**)&d->mvB, &d->mvB_cap, (size_t)n * L * L * R * sizeof(longlong2));
+    if (rc) return rc;
+    longlong2* bufA = (longlong2*)d->mvA;
+    longlong2* bufB = (longlong2*)d->mvB;
+    double2* phase = (double2*)((char*)d->mvA + ba);
+    int* e1 = (int*)((char*)phase + pha);   // [i1][i2]
+    int* e2 = e1 + R * n * n;               // [i1][k3]
+    int* e3 = e2 + R * n * L;               // [k2][k3]
+    int* e4 = e3 + R * L * L;               // [i1][k3]
+    const bool pw = in_mode == MV_IN_PLANEWAVE;
+    const int E = lss_fx_entries(lg, (long long)L * L * L * R, c->num_sms);
+    ProfScope ps(c, s, LSS_PROF_MATVEC, pw ? 6 : 5);
+    FxArgs A{};
+    A.n = (int)n;
+    A.dim = 3;
+    A.N = n * n * n;
+    A.tw = c->fx_tw;
+    A.khat = (const fx_tw*)c->fx_khat;
+    A.ek = c->fx_ek;
+    A.x = x;
+    A.m = c->m;
+    A.y = y;
+    A.uI = uI;
+    A.phase = phase;
+    A.in_mode = in_mode;
+    A.out_mode = out_mode;
+    cudaError_t e = cudaSuccess;
+    if (pw) e = lss_fx_phases(dirs_dev, phase, 3, (int)n, R, c->omega, c->h, s);
+    // lines along x3 at (i1, i2): -> A[i1][i2][k3]
+    A.nlines = (int)(n * n);
+    A.lb = (int)n;
+    A.out = bufA;
+    A.out_r = n * n * L;
+    A.out_a = n * L;
+    A.out_b = L;
+    A.out_s = 1;
+    A.eout = e1;
+    if (!e) e = lss_fx_pass(FX_FWD_IN, lg, E, A, R, s);
+    // lines along x2 at (i1, k3): A -> B[i1][k2][k3]
+    A.nlines = (int)(n * L);
+    A.lb = (int)L;
+    A.in = bufA;
+    A.in_r = n * n * L;
+    A.in_a = n * L;
+    A.in_b = 1;
+    A.in_s = L;
+    A.ein = e1;
+    A.ein_r = n * n;
+    A.ein_a = (int)n;
+    A.ein_b = 0;
+    A.ein_s = 1;
+    A.out = bufB;
+    A.out_r = n * L * L;
+    A.out_a = L * L;
+    A.out_b = 1;
+    A.out_s = L;
+    A.eout = e2;
+    if (!e) e = lss_fx_pass(FX_FWD_MID, lg, E, A, R, s);
+    // lines along x1 at (k2, k3), in place in B
+    A.nlines = (int)(L * L);
+    A.in = bufB;
+    A.in_r = A.out_r = n * L * L;
+    A.in_a = A.out_a = L;
+    A.in_s = A.out_s = L * L;
+    A.ein = e2;
+    A.ein_r = n * L;
+    A.ein_a = 0;
+    A.ein_b = 1;
+    A.ein_s = (int)L;
+    A.eout = e3;
+    if (!e) e = lss_fx_pass(FX_CONV, lg, E, A, R, s);
+    // back along x2 at (i1, k3): B -> A[i1][i2][k3]
+    A.nlines = (int)(n * L);
+    A.in_a = L * L;
+    A.in_s = L;
+    A.ein = e3;
+    A.ein_r = L * L;
+    A.out = bufA;
+    A.out_r = n * n * L;
+    A.out_a = n * L;
+    A.out_s = L;
+    A.eout = e4;
+    if (!e) e = lss_fx_pass(FX_INV_MID, lg, E, A, R, s);
+    // back along x3 at (i1, i2)
+    A.nlines = (int)(n * n);
+    A.lb = (int)n;
+    A.in = bufA;
+    A.in_r = n * n * L;
+    A.in_a = n * L;
+    A.in_b = L;
+    A.in_s = 1;
+    A.ein = e4;
+    A.ein_r = n * L;
+    A.ein_a = (int)L;
+    A.ein_b = 0;
+    A.ein_s = 1;
+    if (!e) e = lss_fx_pass(FX_INV_OUT, lg, E, A, R, s);
+    return lss_check_cuda(c, e, "3D fixed-point matvec launch");
+}
+
 int lss3_matvec(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int out_mode, const double* dirs_dev,
                 double2* uI, cudaStream_t s) {
     Ctx3* d = c->d3;
     const int n = c->n, L = c->L, lg = c->lgL;
+    if (lss_fx_supported(lg)) return matvec3_fx(c, x, y, R, in_mode, out_mode, dirs_dev, uI, s);
     int rc = lss_grow(c, (void**)&d->mvA, &d->mvA_cap, (size_t)n * n * L * R * sizeof(double2));
     if (!rc) rc = lss_grow(c, (void**)&d->mvB, &d->mvB_cap, (size_t)n * L * L * R * sizeof(double2));
     if (rc) return rc;

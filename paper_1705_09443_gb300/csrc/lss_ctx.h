@@ -130,8 +130,13 @@ struct lss_ctx {
 
     // device data
     double* m = nullptr;          // n*n
-    double2* khatT = nullptr;     // L*L, transposed (column k2 contiguous), scaled by omega^2/L^2
+    double2* khatT = nullptr;     // L*L, transposed (column k2 contiguous), scaled by omega^2/L^2 (FP64 operator only)
     double2* tw = nullptr;        // L twiddles exp(-2 pi i k / L)
+    // fixed-point operator (fx_fft.cu; line lengths it does not take keep khatT / tw): twiddle
+    // digits, kernel transform as digits in storage order and its exponent per line
+    void* fx_tw = nullptr;
+    void* fx_khat = nullptr;
+    int* fx_ek = nullptr;
     double2* gam_phys = nullptr;  // (2b+1)^2 x 9 PML stencils (row coefficients)
     double2* gam_aux = nullptr;   // n_samples x b_aux x (2b+1) x 9
     double2* gam_aux_r = nullptr; // the same for the auxiliary PML right of D_i (two fronts)
@@ -276,6 +281,8 @@ int lss_matvec(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int
                const double* dirs_dev, double2* uI, cudaStream_t s);
 int lss_fft_kernel_table(lss_ctx* c, const double2* kc, cudaStream_t s);  // kc: L x L -> khatT
 int lss_fft_configure(lss_ctx* c);
+// the context's fixed-point tables from its kernel transform khat (2D: transposed L x L, 3D: [k2][k3][k1])
+int lss_fx_tables(lss_ctx* c, const double2* khat, cudaStream_t s);
 std::vector<int> lss_fft_col_candidates(const lss_ctx* c);   // admissible column groups (autotuner)
 // slab.cu: chunk tables of every solve plan under the current launch parameters
 int lss_prepare_solve_tables(lss_ctx* c, cudaStream_t s);
