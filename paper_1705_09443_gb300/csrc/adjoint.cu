@@ -34,7 +34,7 @@
 namespace {
 
 constexpr int kTThreads = 256;
-enum TMode { T_A = 0, T_E = 1, T_IF = 2 };
+enum TMode { T_A = 0, T_E = 1 };
 
 __device__ __forceinline__ double2 cfnma_t(double2 a, double2 b, double2 acc) {
     acc.x = fma(-a.x, b.x, acc.x); acc.x = fma(a.y, b.y, acc.x);
@@ -59,8 +59,6 @@ struct TArgs {
     const C* lam;            // T_E couplings lambda', phi', [slab][k][R]
     const C* phi;
     C* X;                    // T_E output: R x n_tot^2 grid, x2 index slowest
-    C* maps;                 // T_IF output: Lambda', Gamma', Phi', each n_slabs x n_tot^2
-    int nch;                 // T_IF: columns per slab side (n_tot)
     C* bg;                   // right-hand sides in global memory when bsm == 0
     long long bstride;
     int bsm;
@@ -99,7 +97,7 @@ __device__ __forceinline__ C bandt(const C* __restrict__ band, int p, const C* x
 }
 
 template <typename T, int MODE, int G>
-__device__ void t_body(const TArgs<cx<T>>& A, const SlabDev& sd, int i, int r, int side, int j, cx<T>* b) {
+__device__ void t_body(const TArgs<cx<T>>& A, const SlabDev& sd, int i, int r, cx<T>* b) {
     using C = cx<T>;
     const int K = A.n_tot, w = sd.w, na = sd.na, bs = sd.bs;
     const int L = cr_levels(K);
@@ -122,42 +120,29 @@ __device__ void t_body(const TArgs<cx<T>>& A, const SlabDev& sd, int i, int r, i
         const int k = e / G, pp = e % G;
         C v = czero<C>();
         if (pp < w) {
-            if (MODE == T_A || MODE == T_E) {
-                const int x1 = sd.s + (pp - na), i2 = k - A.b;
-                if (pp >= na && x1 >= 1 && x1 <= A.n && i2 >= 1 && i2 <= A.n)
-                    v = to_c<C>(A.y[(long long)r * A.n * A.n + (long long)(x1 - 1) * A.n + (i2 - 1)]);
-                if (MODE == T_E) {
-                    const long long vec = (long long)K * A.R;
-                    if (pp == na && i > 0) {   // - H_{[i-1,i]}^T lambda'_{i-1}
-                        const SlabDev sl = A.slabs[i - 1];
-                        const C* cl = A.coef + sl.coef_off;
-                        for (int d = -1; d <= 1; ++d) {
-                            const int kk = k - d;
-                            if (kk >= 0 && kk < K)
-                                v = cfnma_t(cl[(long long)kk * sl.cstride + (sl.w - 1) * 9 + 6 + d + 1],
-                                            A.lam[(long long)(i - 1) * vec + (long long)kk * A.R + r], v);
-                        }
-                    }
-                    if (pp == w - 1 && i < A.n_slabs - 1) {   // - H_{[i+1,i]}^T phi'_{i+1}
-                        const SlabDev sr = A.slabs[i + 1];
-                        const C* crt = A.coef + sr.coef_off;
-                        for (int d = -1; d <= 1; ++d) {
-                            const int kk = k - d;
-                            if (kk >= 0 && kk < K)
-                                v = cfnma_t(crt[(long long)kk * sr.cstride + sr.na * 9 + d + 1],
-                                            A.phi[(long long)(i + 1) * vec + (long long)kk * A.R + r], v);
-                        }
+            const int x1 = sd.s + (pp - na), i2 = k - A.b;
+            if (pp >= na && x1 >= 1 && x1 <= A.n && i2 >= 1 && i2 <= A.n)
+                v = to_c<C>(A.y[(long long)r * A.n * A.n + (long long)(x1 - 1) * A.n + (i2 - 1)]);
+            if (MODE == T_E) {
+                const long long vec = (long long)K * A.R;
+                if (pp == na && i > 0) {   // - H_{[i-1,i]}^T lambda'_{i-1}
+                    const SlabDev sl = A.slabs[i - 1];
+                    const C* cl = A.coef + sl.coef_off;
+                    for (int d = -1; d <= 1; ++d) {
+                        const int kk = k - d;
+                        if (kk >= 0 && kk < K)
+                            v = cfnma_t(cl[(long long)kk * sl.cstride + (sl.w - 1) * 9 + 6 + d + 1],
+                                        A.lam[(long long)(i - 1) * vec + (long long)kk * A.R + r], v);
                     }
                 }
-            } else {
-                const int d = k - j;
-                if (d >= -1 && d <= 1) {
-                    if (side == 0 && pp == na) {   // column j of H_{[i-1,i]}^T
-                        const SlabDev sl = A.slabs[i - 1];
-                        v = A.coef[sl.coef_off + (long long)j * sl.cstride + (sl.w - 1) * 9 + 6 + d + 1];
-                    } else if (side == 1 && pp == w - 1) {   // column j of H_{[i+1,i]}^T
-                        const SlabDev sr = A.slabs[i + 1];
-                        v = A.coef[sr.coef_off + (long long)j * sr.cstride + sr.na * 9 + d + 1];
+                if (pp == w - 1 && i < A.n_slabs - 1) {   // - H_{[i+1,i]}^T phi'_{i+1}
+                    const SlabDev sr = A.slabs[i + 1];
+                    const C* crt = A.coef + sr.coef_off;
+                    for (int d = -1; d <= 1; ++d) {
+                        const int kk = k - d;
+                        if (kk >= 0 && kk < K)
+                            v = cfnma_t(crt[(long long)kk * sr.cstride + sr.na * 9 + d + 1],
+                                        A.phi[(long long)(i + 1) * vec + (long long)kk * A.R + r], v);
                     }
                 }
             }
@@ -252,21 +237,10 @@ __device__ void t_body(const TArgs<cx<T>>& A, const SlabDev& sd, int i, int r, i
             A.a_first[base + (long long)k * A.R] = row(k)[na];
             A.a_last[base + (long long)k * A.R] = row(k)[w - 1];
         }
-    } else if (MODE == T_E) {
+    } else {
         for (int e = tid; e < sd.nl * K; e += nth) {
             const int k = e % K, pp = na + e / K;
             A.X[(long long)r * nt2 + (long long)k * K + sd.s + A.b + (pp - na)] = row(k)[pp];
-        }
-    } else {
-        const int ns = A.n_slabs;
-        for (int k = tid; k < K; k += nth) {
-            const long long o = (long long)k * K + j;
-            if (side == 0) {
-                A.maps[(0LL * ns + i) * nt2 + o] = row(k)[w - 1];
-                A.maps[(1LL * ns + i) * nt2 + o] = row(k)[na];
-            } else {
-                A.maps[(2LL * ns + i) * nt2 + o] = row(k)[na];
-            }
         }
     }
 }
@@ -275,22 +249,13 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(kTThreads) cr_solve_t_kernel(TArgs<cx<T>> A) {
     using C = cx<T>;
     extern __shared__ __align__(16) unsigned char smt[];
-    int i, r = 0, side = 0, j = 0;
-    if (MODE == T_IF) {
-        // blocks: side 0 for slabs 1..l-1, then side 1 for slabs 1..l-2; one column each
-        int t = blockIdx.x;
-        const int n0 = (A.n_slabs - 1) * A.nch;
-        if (t < n0) { i = 1 + t / A.nch; j = t % A.nch; }
-        else { t -= n0; side = 1; i = 1 + t / A.nch; j = t % A.nch; }
-    } else {   // slab-major grid: a slab's right-hand sides share its factor stream in L2
-        i = blockIdx.y;
-        r = blockIdx.x;
-    }
+    // slab-major grid: a slab's right-hand sides share its factor stream in L2
+    const int i = blockIdx.y, r = blockIdx.x;
     const long long cta = (long long)blockIdx.y * gridDim.x + blockIdx.x;
     C* b = A.bsm ? reinterpret_cast<C*>(smt) : A.bg + cta * A.bstride;
     const SlabDev sd = A.slabs[i];
-    if (sd.w <= 16) t_body<T, MODE, 16>(A, sd, i, r, side, j, b);
-    else t_body<T, MODE, 32>(A, sd, i, r, side, j, b);
+    if (sd.w <= 16) t_body<T, MODE, 16>(A, sd, i, r, b);
+    else t_body<T, MODE, 32>(A, sd, i, r, b);
 }
 
 int ldwmax(const lss_ctx* c) {
@@ -350,12 +315,7 @@ int build_maps_t(lss_ctx* c, cudaStream_t s) {
         cudaError_t e = cudaMalloc(&c->iface_t, bytes);
         if (e) return lss_check_cuda(c, e, "transposed interface maps");
     }
-    TArgs<C> A = targs<C>(c, 1);
-    A.maps = (C*)c->iface_t;
-    A.nch = c->n_tot;
-    const int nitems = (c->n_slabs - 1) * c->n_tot + std::max(0, c->n_slabs - 2) * c->n_tot;
-    ProfScope ps(c, s, LSS_PROF_IFACE, 1);
-    int rc = launch_t<T, T_IF>(c, A, dim3(nitems), s);
+    const int rc = lss_iface_maps_t(c, s);
     if (!rc) c->iface_t_valid = true;
     return rc;
 }

@@ -448,6 +448,74 @@ __global__ void __launch_bounds__(256) if_maps_kernel(IfArgs<cx<T>> A) {
     }
 }
 
+// Maps of the transposed sweep from the same columns.  With
+// G_pq = (S_i^{-1})[(p, j'), (q, k)] (p, q = first or last layer of D_i) the
+// transposed subproblem's columns are G transposed, so
+//   Lambda'_i[k][j] = sum_j' G_first,last[j'][k] H_{[i-1,i]}(j, j'),
+//   Gamma'_i with G_first,first, and Phi'_i[k][j] = sum_j' G_last,first[j'][k]
+//   H_{[i+1,i]}(j, j'),
+// couplings tridiagonal in (j, j'): a problem of side 0 gives Gamma'_i and
+// Phi'_i, one of side 1 Lambda'_i.  Bound by memory: W is read and the maps
+// written once, through 32 x 32 tiles transposed in shared memory.  (Solving
+// the transposed subproblems for every column took 98 ms in FP64 at n = 256,
+// this 0.2 ms.)
+constexpr int kMtT = 32;
+template <typename T>
+__global__ void __launch_bounds__(256) if_maps_t_kernel(IfArgs<cx<T>> A) {
+    using C = cx<T>;
+    __shared__ C tile[kMtT + 2][kMtT + 1];   // rows j0 - 1 .. j0 + 32 of W, columns k0 ..
+    const IfProb pr = A.probs[blockIdx.z];
+    const int K = A.K, i = pr.slab, ns = A.n_slabs;
+    const long long nt2 = (long long)K * K;
+    const int k0 = blockIdx.x * kMtT, j0 = blockIdx.y * kMtT;
+    const int tx = threadIdx.x % kMtT, ty = threadIdx.x / kMtT;
+    const int nw = pr.side == 0 ? (i <= ns - 2 ? 2 : 1) : 1;
+    for (int w = 0; w < nw; ++w) {
+        // w = 0: the pinned first layer's rows with slab i-1; 1: the last layer's with slab i+1
+        const C* W = A.W + pr.woff + w * nt2;
+        const SlabDev sn = A.slabs[w == 0 ? i - 1 : i + 1];
+        const C* cf = A.coef + sn.coef_off + (w == 0 ? sn.ll * 9 + 6 : sn.na * 9);
+        C* out = A.maps + ((long long)(pr.side == 1 ? 0 : w == 0 ? 1 : 2) * ns + i) * nt2;
+        if (w) __syncthreads();
+        for (int r = ty; r < kMtT + 2; r += 256 / kMtT) {
+            const int j = j0 - 1 + r, k = k0 + tx;
+            tile[r][tx] = j >= 0 && j < K && k < K ? W[(long long)j * K + k] : czero<C>();
+        }
+        __syncthreads();
+        const int j = j0 + tx;
+        if (j >= K) continue;
+        C h[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) h[d] = cf[(long long)j * sn.cstride + d];
+        for (int r = ty; r < kMtT; r += 256 / kMtT) {
+            const int k = k0 + r;
+            if (k >= K) break;
+            C v = czero<C>();
+#pragma unroll
+            for (int d = 0; d < 3; ++d) v = cfma(tile[tx + d][r], h[d], v);   // (row outside: zero)
+            out[(long long)k * K + j] = v;
+        }
+    }
+}
+
+template <typename T>
+int iface_t_impl(lss_ctx* c, cudaStream_t s) {
+    using C = cx<T>;
+    const int K = c->n_tot;
+    IfArgs<C> A{};
+    A.slabs = c->d_slabs;
+    A.n_slabs = c->n_slabs;
+    A.K = K;
+    A.coef = (const C*)c->coef;
+    A.probs = (const IfProb*)c->ifp_buf;
+    A.W = (C*)c->ifx_buf + c->if_woff;
+    A.maps = (C*)c->iface_t;
+    ProfScope ps(c, s, LSS_PROF_IFACE, 1);
+    const unsigned t = (K + kMtT - 1) / kMtT;
+    if_maps_t_kernel<T><<<dim3(t, t, c->ifp_n), 256, 0, s>>>(A);
+    return lss_check_cuda(c, cudaGetLastError(), "transposed interface maps launch");
+}
+
 template <typename T>
 int iface_impl(lss_ctx* c, cudaStream_t s) {
     using C = cx<T>;
@@ -494,6 +562,7 @@ int iface_impl(lss_ctx* c, cudaStream_t s) {
     A.probs = (const IfProb*)c->ifp_buf;
     A.X = (C*)c->ifx_buf;
     A.W = A.X + xoff;
+    c->if_woff = xoff;
     A.maps = (C*)c->iface;
     A.psi = c->fronts == 2;
     const size_t sh = sizeof(C) * ((size_t)3 * gmax * gmax + (size_t)8 * gmax);
@@ -567,6 +636,10 @@ int iface_impl(lss_ctx* c, cudaStream_t s) {
 }
 
 }  // namespace
+
+int lss_iface_maps_t(lss_ctx* c, cudaStream_t s) {
+    return c->prec == LSS_FP64 ? iface_t_impl<double>(c, s) : iface_t_impl<float>(c, s);
+}
 
 int lss_iface_maps(lss_ctx* c, cudaStream_t s) {
     return c->prec == LSS_FP64 ? iface_impl<double>(c, s) : iface_impl<float>(c, s);

@@ -164,6 +164,7 @@ struct lss_ctx {
     void* gr_buf = nullptr; size_t gr_cap = 0;         // -omega^2 K mu for the medium gradient
     void* hz_buf = nullptr; size_t hz_cap = 0;         // direct Helmholtz solve: beta^* f and u on the grid
     void* ifx_buf = nullptr; size_t ifx_cap = 0;       // interface-map column blocks (all slabs, both sides)
+    long long if_woff = 0;                             // entries of ifx_buf before the kept layers W (they stay until the next factorization)
     void* ifp_buf = nullptr; size_t ifp_cap = 0;       // interface-map problem table
     int ifp_n = 0;                                     // problems uploaded to ifp_buf
     // slab-solve chunk tables: key (first/last layers only, stage entries, chunks
@@ -301,6 +302,8 @@ int lss_sweep(lss_ctx* c, const double2* r, double2* y, int R, cudaStream_t s);
 int lss_slab_apply(lss_ctx* c, int slab, const double2* v, double2* w, int R, cudaStream_t s);
 // iface.cu: interface maps Lambda, Gamma, Phi of every slab (all columns at once)
 int lss_iface_maps(lss_ctx* c, cudaStream_t s);
+// the transposed sweep's maps into iface_t, from what lss_iface_maps left in ifx_buf
+int lss_iface_maps_t(lss_ctx* c, cudaStream_t s);
 // the three interface recurrences with the maps at `maps` (Lambda, Gamma, Phi blocks)
 int lss_recurrences(lss_ctx* c, const void* maps, void* lam, void* phi, const void* a_first, const void* a_last,
                     int R, cudaStream_t s);
