@@ -308,6 +308,10 @@ int lss_iface_maps_t(lss_ctx* c, cudaStream_t s);
 int lss_recurrences(lss_ctx* c, const void* maps, void* lam, void* phi, const void* a_first, const void* a_last,
                     int R, cudaStream_t s);
 
+// recur.cu: the same for more than 8 right-hand sides that no cluster holds
+int lss_recur_wide(lss_ctx* c, const void* maps, void* lam, void* phi, const void* a_first, const void* a_last,
+                   int R, cudaStream_t s);
+
 // adjoint.cu: the transposed preconditioner P^T = Q^T Sweep^T E^T
 int lss_sweep_t(lss_ctx* c, const double2* y, double2* r, int R, cudaStream_t s);
 // builds the transposed interface maps now if the factorization changed (the

@@ -925,97 +925,9 @@ __global__ void __launch_bounds__(kSolveThreads) cr_solve_kernel(CrArgs<cx<T>> A
 
 // ---------------------------------------------------------------- interface recurrences
 // Grid-wide version (cooperative launch, bounded grid barrier): the fallback
-// when the vectors or rows do not fit the cluster kernel below.
-// Tiles of the grid-synchronised recurrence: each step is a product of an
-// n_tot x n_tot map with the n_tot x R block of current vectors; a CTA forms a
-// kGtR x kGtC tile of it over K chunks of kGtK staged in shared memory
-// (coalesced loads of map rows and vector rows, the next chunk loaded into
-// registers while the current one is multiplied).  Each thread owns four rows
-// of one column, so a vector entry read from shared memory serves four
-// products and the map entries are read as broadcasts.
-// Tiles of TR = 64 rows (4 per thread) when a step has enough of them,
-// else TR = 32 (2 per thread).  The K chunks stream into a ring of kGtS
-// shared-memory stages by cp.async copies issued kGtS - 1 chunks ahead (many
-// bytes in flight per SM: the maps come from DRAM at every step).
-constexpr int kGtC = 16, kGtK = 32, kGtS = 4;
-
-
-// entries of one ring stage: the map tile (TR rows, kGtK + 2 per row) and
-// the vector tile (kGtK rows, kGtC + 1 per row)
-template <int TR>
-constexpr int gt_stage_ent() { return TR * (kGtK + 2) + kGtK * (kGtC + 1); }
-
-template <typename T, int TR>
-__device__ __forceinline__ void recur_tile(const cx<T>* __restrict__ M, const cx<T>* x, const cx<T>* base,
-                                           cx<T>* out, int n_tot, int R, int rt, int ct, cx<T>* ring) {
-    using C = cx<T>;
-    constexpr int RPT = TR / 16;                  // rows per thread
-    constexpr int LA = TR * kGtK / 256;           // map entries a thread copies per chunk
-    constexpr int LB = kGtK * kGtC / 256;         // vector entries a thread copies per chunk
-    constexpr int SE = gt_stage_ent<TR>();
-    static_assert(TR * kGtK % 256 == 0 && kGtK * kGtC % 256 == 0, "a chunk must split evenly over the threads");
-    const int tid = threadIdx.x;
-    const int ty = tid / kGtC, tx = tid % kGtC;   // rows RPT ty .. RPT ty + RPT - 1, column tx
-    const int nch = (n_tot + kGtK - 1) / kGtK;
-    auto issue = [&](int ch) {
-        if (ch < nch) {
-            C* As = ring + (ch % kGtS) * SE;
-            C* Bs = As + TR * (kGtK + 2);
-            const int k0 = ch * kGtK;
-#pragma unroll
-            for (int u = 0; u < LA; ++u) {
-                const int e = tid + 256 * u;
-                const int a = e / kGtK, kk = e % kGtK;
-                const int gr = rt * TR + a, gk = k0 + kk;
-                const bool ok = gr < n_tot && gk < n_tot;
-                cp_async_entry(As + a * (kGtK + 2) + kk, ok ? M + (long long)gr * n_tot + gk : M, ok);
-            }
-#pragma unroll
-            for (int u = 0; u < LB; ++u) {
-                const int e = tid + 256 * u;
-                const int kk = e / kGtC, c = e % kGtC;
-                const int gk = k0 + kk, gc = ct * kGtC + c;
-                const bool ok = gk < n_tot && gc < R;
-                cp_async_entry(Bs + kk * (kGtC + 1) + c, ok ? x + (long long)gk * R + gc : x, ok);
-            }
-        }
-        cp_async_commit();   // (an empty group past the last chunk keeps the count uniform)
-    };
-    C acc[RPT];
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) acc[i] = czero<C>();
-#pragma unroll
-    for (int q = 0; q < kGtS - 1; ++q) issue(q);
-    for (int ch = 0; ch < nch; ++ch) {
-        cp_async_wait<kGtS - 2>();   // chunk ch has landed (this thread's copies)
-        __syncthreads();             // ... and every thread's
-        const C* As = ring + (ch % kGtS) * SE;
-        const C* Bs = As + TR * (kGtK + 2);
-#pragma unroll 8
-        for (int kk = 0; kk < kGtK; ++kk) {
-            const C bv = Bs[kk * (kGtC + 1) + tx];
-#pragma unroll
-            for (int i = 0; i < RPT; ++i) acc[i] = cfma(As[(RPT * ty + i) * (kGtK + 2) + kk], bv, acc[i]);
-        }
-        __syncthreads();             // the stage of chunk ch may be refilled
-        issue(ch + kGtS - 1);
-    }
-    cp_async_wait<0>();
-    const int col = ct * kGtC + tx;
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-        const int row = rt * TR + RPT * ty + i;
-        if (row < n_tot && col < R) {
-            const long long e = (long long)row * R + col;
-            out[e] = base[e] - acc[i];
-        }
-    }
-}
-
-// Few right-hand sides (R <= RM, RM in 1, 2, 4, 8): a 16-column tile would
-// spend most of its multiply-adds on absent columns (on FP64, where the pipe
-// is the bound, up to 16 times the work), so a tile is TR rows instead, two
-// per warp: lanes stride over k (coalesced map rows, the vector entries shared
+// when the vectors or rows do not fit the cluster kernel below, for few
+// right-hand sides (R <= RM, RM in 1, 2, 4, 8; more go to recur.cu): a task is TR rows of every column, two rows per
+// warp: lanes stride over k (coalesced map rows, the vector entries shared
 // by the warp's two rows), then a shuffle reduction per row and column.
 template <typename T, int RM>
 __device__ __forceinline__ void recur_rows(const cx<T>* __restrict__ M, const cx<T>* x, const cx<T>* base,
@@ -1068,38 +980,30 @@ __device__ __forceinline__ void recur_rows(const cx<T>* __restrict__ M, const cx
     }
 }
 
-// One task of a recurrence step: tile (rt, ct) of out = base - M x.  RM = 0:
-// TR x kGtC tiles staged through the ring; RM > 0: TR-row tiles, every column.
-template <typename T, int TR, int RM>
-__device__ __forceinline__ void recur_task(const cx<T>* __restrict__ M, const cx<T>* x, const cx<T>* base,
-                                           cx<T>* out, int n_tot, int R, int rt, int ct, cx<T>* ring) {
-    if constexpr (RM == 0)
-        recur_tile<T, TR>(M, x, base, out, n_tot, R, rt, ct, ring);
-    else
-        recur_rows<T, RM>(M, x, base, out, n_tot, R, rt * TR, min(TR, n_tot - rt * TR));
-}
-
-template <int RM>
-__host__ __device__ constexpr int recur_col_tiles(int R) { return RM ? 1 : (R + kGtC - 1) / kGtC; }
-
 // Recurrences of all slabs with one cooperative grid when the vectors do not
 // fit the cluster kernels (many right-hand sides): lambda and mu, then phi,
 // one step per slab, a grid barrier between steps; the tiles of a step are
 // spread over the CTAs.
-template <typename T, int TR, int RM>
+constexpr int kRowsTR = 16;   // rows per task
+
+// One task of a recurrence step: rows rt kRowsTR .. of out = base - M x.
+template <typename T, int RM>
+__device__ __forceinline__ void recur_task(const cx<T>* __restrict__ M, const cx<T>* x, const cx<T>* base,
+                                           cx<T>* out, int n_tot, int R, int rt) {
+    recur_rows<T, RM>(M, x, base, out, n_tot, R, rt * kRowsTR, min(kRowsTR, n_tot - rt * kRowsTR));
+}
+
+template <typename T, int RM>
 __global__ void __launch_bounds__(256) recur_grid_kernel(int n_slabs, int n_tot, int R,
                                                          const cx<T>* __restrict__ iface,
                                                          const cx<T>* __restrict__ a_first,
                                                          const cx<T>* __restrict__ a_last, cx<T>* lam, cx<T>* phi,
                                                          unsigned* bar, int* err) {
     using C = cx<T>;
-    extern __shared__ __align__(16) unsigned char gts[];
-    C* ring = reinterpret_cast<C*>(gts);   // kGtS stages of gt_stage_ent<TR>() entries
     unsigned nbar = 0;                     // grid barriers passed (the arrival counter starts at zero)
     const long long nt2 = (long long)n_tot * n_tot;
     const long long vec = (long long)n_tot * R;
-    const int nrt = (n_tot + TR - 1) / TR, nct = recur_col_tiles<RM>(R);
-    const int ntile = nrt * nct;
+    const int ntile = (n_tot + kRowsTR - 1) / kRowsTR;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < vec;
          e += (long long)gridDim.x * blockDim.x)
         lam[e] = a_last[e];
@@ -1109,18 +1013,18 @@ __global__ void __launch_bounds__(256) recur_grid_kernel(int n_slabs, int n_tot,
         for (int task = blockIdx.x; task < nwhich * ntile; task += gridDim.x) {   // uniform per CTA
             const int which = task / ntile, t = task % ntile;
             if (which == 0)   // mu_i = first(a_i) - Gamma_i lambda_{i-1}
-                recur_task<T, TR, RM>(iface + (1LL * n_slabs + i) * nt2, lp, a_first + (long long)i * vec,
-                              phi + (long long)i * vec, n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(iface + (1LL * n_slabs + i) * nt2, lp, a_first + (long long)i * vec,
+                              phi + (long long)i * vec, n_tot, R, t);
             else              // lambda_i = last(a_i) - Lambda_i lambda_{i-1}
-                recur_task<T, TR, RM>(iface + (long long)i * nt2, lp, a_last + (long long)i * vec,
-                              lam + (long long)i * vec, n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(iface + (long long)i * nt2, lp, a_last + (long long)i * vec,
+                              lam + (long long)i * vec, n_tot, R, t);
         }
         grid_barrier_count(bar, (++nbar) * gridDim.x, err);
     }
     for (int i = n_slabs - 2; i >= 1; --i) {   // phi_i = mu_i - Phi_i phi_{i+1}
         for (int task = blockIdx.x; task < ntile; task += gridDim.x)
-            recur_task<T, TR, RM>(iface + (2LL * n_slabs + i) * nt2, phi + (long long)(i + 1) * vec,
-                          phi + (long long)i * vec, phi + (long long)i * vec, n_tot, R, task / nct, task % nct, ring);
+            recur_task<T, RM>(iface + (2LL * n_slabs + i) * nt2, phi + (long long)(i + 1) * vec,
+                          phi + (long long)i * vec, phi + (long long)i * vec, n_tot, R, task);
         grid_barrier_count(bar, (++nbar) * gridDim.x, err);
     }
 }
@@ -1139,20 +1043,17 @@ __global__ void __launch_bounds__(256) recur_grid_kernel(int n_slabs, int n_tot,
 //   back:    phi_i = mu_i - Phi_i phi_{i+1} (i < c),  lambda_i = nu_i - Lambda_i lambda_{i-1} (i > c)
 // Both fronts advance in the same grid step, so the dependent steps are about
 // half of the one-front recurrences'.
-template <typename T, int TR, int RM>
+template <typename T, int RM>
 __global__ void __launch_bounds__(256) recur_grid2_kernel(int n_slabs, int mid, int n_tot, int R,
                                                           const cx<T>* __restrict__ iface,
                                                           const cx<T>* __restrict__ a_first,
                                                           const cx<T>* __restrict__ a_last, cx<T>* lam, cx<T>* phi,
                                                           unsigned* bar, int* err) {
     using C = cx<T>;
-    extern __shared__ __align__(16) unsigned char gts[];
-    C* ring = reinterpret_cast<C*>(gts);   // kGtS stages of gt_stage_ent<TR>() entries
     unsigned nbar = 0;                     // grid barriers passed (the arrival counter starts at zero)
     const long long nt2 = (long long)n_tot * n_tot;
     const long long vec = (long long)n_tot * R;
-    const int nrt = (n_tot + TR - 1) / TR, nct = recur_col_tiles<RM>(R);
-    const int ntile = nrt * nct;
+    const int ntile = (n_tot + kRowsTR - 1) / kRowsTR;
     const int ns = n_slabs, c = mid;
     const C* LAM = iface;
     const C* GAM = iface + (long long)ns * nt2;
@@ -1178,15 +1079,13 @@ __global__ void __launch_bounds__(256) recur_grid2_kernel(int n_slabs, int mid, 
             const int t = task % ntile;
             if (!onL) which += 2;
             if (which == 0)
-                recur_task<T, TR, RM>(LAM + iL * nt2, V(lam, iL - 1), Vc(a_last, iL), V(lam, iL), n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(LAM + iL * nt2, V(lam, iL - 1), Vc(a_last, iL), V(lam, iL), n_tot, R, t);
             else if (which == 1)
-                recur_task<T, TR, RM>(GAM + iL * nt2, V(lam, iL - 1), Vc(a_first, iL), V(phi, iL), n_tot, R, t / nct,
-                              t % nct, ring);
+                recur_task<T, RM>(GAM + iL * nt2, V(lam, iL - 1), Vc(a_first, iL), V(phi, iL), n_tot, R, t);
             else if (which == 2)
-                recur_task<T, TR, RM>(PHI + iR * nt2, V(phi, iR + 1), Vc(a_first, iR), V(phi, iR), n_tot, R, t / nct,
-                              t % nct, ring);
+                recur_task<T, RM>(PHI + iR * nt2, V(phi, iR + 1), Vc(a_first, iR), V(phi, iR), n_tot, R, t);
             else
-                recur_task<T, TR, RM>(PSI + iR * nt2, V(phi, iR + 1), Vc(a_last, iR), V(lam, iR), n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(PSI + iR * nt2, V(phi, iR + 1), Vc(a_last, iR), V(lam, iR), n_tot, R, t);
         }
         grid_barrier_count(bar, (++nbar) * gridDim.x, err);
     }
@@ -1195,18 +1094,18 @@ __global__ void __launch_bounds__(256) recur_grid2_kernel(int n_slabs, int mid, 
         for (int task = blockIdx.x; task < 2 * ntile; task += gridDim.x) {
             const int t = task % ntile;
             if (task < ntile)
-                recur_task<T, TR, RM>(GAM + c * nt2, V(lam, c - 1), Vc(a_first, c), V(phi, c), n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(GAM + c * nt2, V(lam, c - 1), Vc(a_first, c), V(phi, c), n_tot, R, t);
             else
-                recur_task<T, TR, RM>(LAM + c * nt2, V(lam, c - 1), Vc(a_last, c), V(lam, c), n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(LAM + c * nt2, V(lam, c - 1), Vc(a_last, c), V(lam, c), n_tot, R, t);
         }
         grid_barrier_count(bar, (++nbar) * gridDim.x, err);
     }
     for (int task = blockIdx.x; task < 2 * ntile; task += gridDim.x) {
         const int t = task % ntile;
         if (task < ntile)
-            recur_task<T, TR, RM>(PHI + c * nt2, V(phi, c + 1), V(phi, c), V(phi, c), n_tot, R, t / nct, t % nct, ring);
+            recur_task<T, RM>(PHI + c * nt2, V(phi, c + 1), V(phi, c), V(phi, c), n_tot, R, t);
         else
-            recur_task<T, TR, RM>(PSI + c * nt2, V(phi, c + 1), V(lam, c), V(lam, c), n_tot, R, t / nct, t % nct, ring);
+            recur_task<T, RM>(PSI + c * nt2, V(phi, c + 1), V(lam, c), V(lam, c), n_tot, R, t);
     }
     grid_barrier_count(bar, (++nbar) * gridDim.x, err);
     for (int st = 0; st < S; ++st) {   // both fronts back toward the boundaries
@@ -1217,9 +1116,9 @@ __global__ void __launch_bounds__(256) recur_grid2_kernel(int n_slabs, int mid, 
             const int t = task % ntile;
             const bool left = onL && task < ntile;
             if (left)
-                recur_task<T, TR, RM>(PHI + iL * nt2, V(phi, iL + 1), V(phi, iL), V(phi, iL), n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(PHI + iL * nt2, V(phi, iL + 1), V(phi, iL), V(phi, iL), n_tot, R, t);
             else
-                recur_task<T, TR, RM>(LAM + iR * nt2, V(lam, iR - 1), V(lam, iR), V(lam, iR), n_tot, R, t / nct, t % nct, ring);
+                recur_task<T, RM>(LAM + iR * nt2, V(lam, iR - 1), V(lam, iR), V(lam, iR), n_tot, R, t);
         }
         grid_barrier_count(bar, (++nbar) * gridDim.x, err);
     }
@@ -2542,40 +2441,27 @@ int launch_recur(lss_ctx* c, const cx<T>* ifc, cx<T>* lam, cx<T>* phi, const cx<
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(s, &cap);
     if (cap != cudaStreamCaptureStatusNone) return LSS_ERR_UNSUPPORTED;
-    // tiles of the widest step (lambda and mu with one front, both fronts' two
-    // products with two): with up to 8 right-hand sides, 16-row tiles of every
-    // column (recur_rows); else 64 x 16 tiles when they cover at least half the
-    // SMs (two 32-row tiles on one SM take longer than one 64-row tile), else 32 x 16
-    const long long prods = two ? 4 : 2;
-    const int RM = R == 1 ? 1 : R == 2 ? 2 : R <= 4 ? 4 : R <= 8 ? 8 : 0;
-    const long long nct = RM ? 1 : (R + kGtC - 1) / kGtC;
-    const int TR = RM ? 16 : 2 * prods * ((c->n_tot + 63) / 64) * nct >= c->num_sms ? 64 : 32;
-    const size_t smem = RM ? 0 : (size_t)kGtS * (TR == 64 ? gt_stage_ent<64>() : gt_stage_ent<32>()) * sizeof(C);
-    const int var = RM ? 2 + (RM == 1 ? 0 : RM == 2 ? 1 : RM == 4 ? 2 : 3) : TR == 64;
+    if (R > 8) return lss_recur_wide(c, ifc, lam, phi, a_first, a_last, R, s);
+    const int var = R == 1 ? 0 : R == 2 ? 1 : R <= 4 ? 2 : 3;
     using KernPtr = const void*;
-    const KernPtr k1[6] = {(KernPtr)recur_grid_kernel<T, 32, 0>, (KernPtr)recur_grid_kernel<T, 64, 0>,
-                           (KernPtr)recur_grid_kernel<T, 16, 1>, (KernPtr)recur_grid_kernel<T, 16, 2>,
-                           (KernPtr)recur_grid_kernel<T, 16, 4>, (KernPtr)recur_grid_kernel<T, 16, 8>};
-    const KernPtr k2[6] = {(KernPtr)recur_grid2_kernel<T, 32, 0>, (KernPtr)recur_grid2_kernel<T, 64, 0>,
-                           (KernPtr)recur_grid2_kernel<T, 16, 1>, (KernPtr)recur_grid2_kernel<T, 16, 2>,
-                           (KernPtr)recur_grid2_kernel<T, 16, 4>, (KernPtr)recur_grid2_kernel<T, 16, 8>};
+    const KernPtr k1[4] = {(KernPtr)recur_grid_kernel<T, 1>, (KernPtr)recur_grid_kernel<T, 2>,
+                           (KernPtr)recur_grid_kernel<T, 4>, (KernPtr)recur_grid_kernel<T, 8>};
+    const KernPtr k2[4] = {(KernPtr)recur_grid2_kernel<T, 1>, (KernPtr)recur_grid2_kernel<T, 2>,
+                           (KernPtr)recur_grid2_kernel<T, 4>, (KernPtr)recur_grid2_kernel<T, 8>};
     const void* k = two ? k2[var] : k1[var];
     int grid_now;
     {
         std::lock_guard<std::mutex> lock(lss_config_mutex());
         long long& g = lss_dev_cache(k, 0);   // co-resident CTAs on this device
         if (!g) {
-            if (smem) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e) return lss_check_cuda(c, e, "recurrence attribute");
-            }
             int per = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 256, smem);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 256, 0);
             g = (long long)std::max(1, per) * c->num_sms;
         }
         grid_now = (int)g;
     }
-    const long long tiles = prods * ((c->n_tot + TR - 1) / TR) * nct;
+    // tasks of the widest step: lambda and mu with one front, both fronts' two products with two
+    const long long tiles = (two ? 4 : 2) * ((c->n_tot + kRowsTR - 1) / kRowsTR);
     int nb = (int)std::min<long long>(grid_now, std::max<long long>(1, tiles));
     int nsl = c->n_slabs, nt = c->n_tot, mid = c->mid;
     unsigned* bar = c->d_bar;
@@ -2585,10 +2471,10 @@ int launch_recur(lss_ctx* c, const cx<T>* ifc, cx<T>* lam, cx<T>* phi, const cx<
     if (e) return lss_check_cuda(c, e, "recurrence barrier");
     if (two) {
         void* args[] = {&nsl, &mid, &nt, &R, &ifc, (void*)&a_first, (void*)&a_last, &lam, &phi, &bar, &err};
-        e = cudaLaunchCooperativeKernel(k, dim3(nb), dim3(256), args, smem, s);
+        e = cudaLaunchCooperativeKernel(k, dim3(nb), dim3(256), args, 0, s);
     } else {
         void* args[] = {&nsl, &nt, &R, &ifc, (void*)&a_first, (void*)&a_last, &lam, &phi, &bar, &err};
-        e = cudaLaunchCooperativeKernel(k, dim3(nb), dim3(256), args, smem, s);
+        e = cudaLaunchCooperativeKernel(k, dim3(nb), dim3(256), args, 0, s);
     }
     return lss_check_cuda(c, e, "recurrence launch");
 }
