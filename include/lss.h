@@ -36,11 +36,10 @@
  * Environment switches (read at each call; each selects between two exact
  * implementations of the same operation, for comparison and testing):
  *  - LSS_SLAB_SOLVE=cr: 2D slab solves always by the block cyclic reduction
- *    (default: the 16-wide slabs of solves with R >= 16 by the block LU).
+ *    (default: in mixed precision the 16-wide slabs of solves with R >= 16 by
+ *    the block LU).
  *  - LSS_BATCH_THREADS=1: a batch context solves each instance on its own
  *    host thread (default: one lockstep Krylov driver for all instances).
- *  - LSS_SOLVE_NR=2: two right-hand sides per cyclic-reduction CTA on 16-wide
- *    slabs from the start (default: the autotuner decides).
  *  - LSS_TC_UPDATE=0: the 3D mixed factorization's rank updates on CUDA
  *    cores (default: 3xTF32 tcgen05 tensor cores).
  */
@@ -328,19 +327,14 @@ int lss_set_graphs(lss_ctx *c, int enable);
 /*
  * lss_autotune - pick launch parameters for R right-hand sides by timing this
  * context's own operations (CUDA events, a few runs per candidate): the FFT
- * column group of the LS operator, the slab-solve shared-memory plan (ring
- * stages; right-hand sides in shared or global memory) and the recurrence's
- * ring depth.  2D grids only (LSS_ERR_UNSUPPORTED on a 3D context).  None of them changes any result (same arithmetic, same order),
+ * column group of the LS operator and the recurrence's ring depth (the slab
+ * solves size themselves).  2D grids only (LSS_ERR_UNSUPPORTED on a 3D context).  None of them changes any result (same arithmetic, same order),
  * so later solves agree bit for bit with untuned ones; only their speed
  * changes.  Requires a factored context; allocates and frees two vectors;
  * blocks the host.  On a batch: every instance.  The paper has no
  * counterpart (launch configuration only).
- *   chosen  host, 7 ints (may be NULL): column group, right-hand sides in
- *           global memory (0) or automatic (-1), ring stages (0 = automatic),
- *           recurrence stages, ring stages of the 32-wide slabs' launches
- *           (0 = as the others), slab solves within half the shared memory
- *           so that two CTAs share an SM (1) or not (0), right-hand sides
- *           per slab-solve CTA on 16-wide slabs (1 or 2)
+ *   chosen  host, 7 ints (may be NULL): column group, -1, 0, recurrence
+ *           stages, 0, 0, 1 (the constants: the slab solves' automatic choice)
  */
 int lss_autotune(lss_ctx *c, int R, int *chosen, void *stream);
 

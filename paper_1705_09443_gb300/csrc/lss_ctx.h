@@ -167,9 +167,9 @@ struct lss_ctx {
     long long if_woff = 0;                             // entries of ifx_buf before the kept layers W (they stay until the next factorization)
     void* ifp_buf = nullptr; size_t ifp_cap = 0;       // interface-map problem table
     int ifp_n = 0;                                     // problems uploaded to ifp_buf
-    // slab-solve chunk tables: key (first/last layers only, stage entries, chunks
-    // of 16-wide blocks, chunks of 32-wide blocks) and two device arrays per key
-    std::vector<std::array<long long, 4>> chunk_keys;
+    // chunk tables of lss_apply_slab: key (stage entries, chunks of 16-wide
+    // blocks, chunks of 32-wide blocks) and two device arrays per key
+    std::vector<std::array<long long, 3>> chunk_keys;
     std::vector<void*> chunk_dev;
     int num_sms = 0;
 
@@ -182,11 +182,6 @@ struct lss_ctx {
     // launch parameters picked by lss_autotune (0 / -1: the built-in choice)
     struct Tune {
         int fft_C = 0;        // columns per CTA of the FFT column pass
-        int solve_bsm = -1;   // 0: slab-solve right-hand sides in global memory even when they fit shared
-        int solve_nst = 0;    // slab-solve ring stages (the stages then share the free shared memory)
-        int solve_nst_w = 0;  // the same for launches of 32-wide slabs only (0: as solve_nst)
-        int solve_half = 0;   // 1: slab solves keep to half the shared memory (two CTAs per SM)
-        int solve_nr = 1;     // right-hand sides per slab-solve CTA on 16-wide slabs (1 or 2)
         int rec_nb = 0;       // ring stages of the TMA recurrence
     } tune;
 
@@ -285,8 +280,6 @@ int lss_fft_configure(lss_ctx* c);
 // the context's fixed-point tables from its kernel transform khat (2D: transposed L x L, 3D: [k2][k3][k1])
 int lss_fx_tables(lss_ctx* c, const double2* khat, cudaStream_t s);
 std::vector<int> lss_fft_col_candidates(const lss_ctx* c);   // admissible column groups (autotuner)
-// slab.cu: chunk tables of every solve plan under the current launch parameters
-int lss_prepare_solve_tables(lss_ctx* c, cudaStream_t s);
 // slab.cu: at least n - 1 auxiliary streams (with events) and the fork event
 int lss_ensure_aux(lss_ctx* c, size_t n);
 

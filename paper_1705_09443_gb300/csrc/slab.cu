@@ -41,6 +41,7 @@
 
 #include <cooperative_groups.h>
 
+#include "cr_cluster.h"
 #include "lss_common.cuh"
 #include "lss_ctx.h"
 #include "lss3d.h"
@@ -450,10 +451,11 @@ __global__ void __launch_bounds__(kWideThreads) cr_evenw_kernel(const SlabDev* _
 }
 
 // ---------------------------------------------------------------- slab solves
-// One kernel for the three uses of T~_i:
-//   CR_A    sweep, first pass: a_i = T~_i f_i, first and last layers kept;
-//   CR_E    sweep, second pass: T~_i (f_i - H lambda_{i-1} - H phi_{i+1}) on D_i;
-//   CR_TEST T~_i applied to given vectors (lss_apply_slab).
+// The sweep's two passes,
+//   CR_A    a_i = T~_i f_i, first and last layers kept,
+//   CR_E    T~_i (f_i - H lambda_{i-1} - H phi_{i+1}) on D_i,
+// run on clusters (cr_cluster.cu) or by the block LU below.  The kernel here
+// applies T~_i to given vectors (lss_apply_slab).
 // A CTA solves one right-hand side of one slab, held in shared memory (or
 // per-CTA global scratch when it does not fit), block row k at b + k * G.  The
 // factors stream through a ring of shared-memory stages in the order the solve
@@ -465,7 +467,7 @@ __global__ void __launch_bounds__(kWideThreads) cr_evenw_kernel(const SlabDev* _
 // barrier after each chunk frees its stage.  Lanes are grouped by G (16 when
 // the slab is at most 16 layers wide, else 32): lane p of a group owns layer p
 // of one block row.
-enum CrMode { CR_A = 0, CR_E = 1, CR_TEST = 2 };
+enum CrMode { CR_A = 0, CR_E = 1 };
 enum CrPhase { PH_FODD = 0, PH_FEVEN = 1, PH_TOP = 2, PH_BODD = 3, PH_B0 = 4 };
 
 // One chunk of a solve: phase, level, block rows [r0, r1) of the phase, and the
@@ -489,7 +491,7 @@ struct CrArgs {
     const C* phi;
     double2* y;              // CR_E output, R x n^2 (or R x n_tot^2 when y_grid)
     int y_grid;              // CR_E: write every point of D_i on the grid (x2 slowest) instead of I
-    int slab;                // CR_TEST
+    int slab;                // lss_apply_slab
     const double2* v_in;     // R x (layers of D_i) x n_tot
     double2* w_out;
     const CrChunk* tab16;    // chunk tables for 16- and 32-wide blocks
@@ -565,17 +567,17 @@ __device__ __forceinline__ C mv_part(const C* M, int p, const C* x, int a0) {
 // Phases whose 32-wide block rows are split over four warps, and the most
 // block rows such a chunk holds (4 x 6 warp tasks: two per warp)
 constexpr int kSplitRows = 6;
-__host__ __device__ __forceinline__ bool cr_split_phase(int G, int kind, int l, bool part) {
-    return G == 32 && !(kind == PH_FEVEN && l == 0) && !(kind == PH_B0 && part);
+__host__ __device__ __forceinline__ bool cr_split_phase(int G, int kind, int l) {
+    return G == 32 && !(kind == PH_FEVEN && l == 0);
 }
 
 // The chunk sequence of one solve (host side): phases FODD(l), FEVEN(l) for
 // l = 0..L-1, TOP, BODD(l) for l = L-1..1, B0; each phase's block rows in chunks
 // of at most min(2 x lane groups, stage / row size) rows.
-std::vector<CrChunk> cr_chunk_table(int K, int G, bool part, int stage_ent, int groups) {
+std::vector<CrChunk> cr_chunk_table(int K, int G, int stage_ent, int groups) {
     std::vector<CrChunk> out;
     const int L = cr_levels(K), bs = G * G;
-    const long long t0 = cr_t0_off(K, bs), p0 = cr_p0_off(K, bs, G);
+    const long long t0 = cr_t0_off(K, bs);
     const CrLevelOffs top = cr_level(K, L);
     for (int ph = 0; ph < 3 * L + 1; ++ph) {
         int kind, l, rb;
@@ -596,10 +598,10 @@ std::vector<CrChunk> cr_chunk_table(int K, int G, bool part, int stage_ent, int 
             case PH_FODD: case PH_TOP: row = bs; break;
             case PH_FEVEN: row = l == 0 ? 6 * G : 2 * bs; break;
             case PH_BODD: row = 2 * bs; break;
-            default: row = 6 * G + (part ? 2 * G : bs);
+            default: row = 6 * G + bs;
         }
         int rpc = std::max(1, std::min(2 * groups, stage_ent / row));
-        if (cr_split_phase(G, kind, l, part)) rpc = std::min(rpc, kSplitRows);
+        if (cr_split_phase(G, kind, l)) rpc = std::min(rpc, kSplitRows);
         const CrLevelOffs lv = cr_level(K, l);
         for (int r0 = 0; r0 < rb; r0 += rpc) {
             const int r1 = std::min(rb, r0 + rpc), nr = r1 - r0;
@@ -615,8 +617,8 @@ std::vector<CrChunk> cr_chunk_table(int K, int G, bool part, int stage_ent, int 
                 default:
                     ch.src = t0 + ((long long)(K + 1) / 2 + r0) * 6 * G;
                     ch.ent = nr * 6 * G;
-                    if (part) { ch.src2 = p0 + 2LL * r0 * G; ch.ent2 = 2 * nr * G; }
-                    else { ch.src2 = (cr_level(K, 0).dinv + r0) * bs; ch.ent2 = nr * bs; }
+                    ch.src2 = (cr_level(K, 0).dinv + r0) * bs;
+                    ch.ent2 = nr * bs;
             }
             out.push_back(ch);
         }
@@ -624,13 +626,10 @@ std::vector<CrChunk> cr_chunk_table(int K, int G, bool part, int stage_ent, int 
     return out;
 }
 
-// One CTA solves slab i's subproblem for NR right-hand sides r, r+1, ..,
-// each factor chunk serving all of them (NR = 2 only with 16-wide blocks);
-// b holds the NR right-hand sides one after another.
-template <typename C, int MODE, int G, int NR>
+// One CTA solves slab i's subproblem for right-hand side r, held in b.
+template <typename C, int G>
 __device__ __forceinline__ void cr_body(const CrArgs<C>& A, const SlabDev& sd, int i, int r, C* b, C* tb, C* ring,
                                         uint64_t* full, int4* desc, const CrLv* lv, bool& ok) {
-    static_assert(NR == 1 || G == 16, "several right-hand sides per CTA with 16-wide blocks only");
     const int K = A.n_tot, w = sd.w, bs = sd.bs, na = sd.na;
     const int tid = threadIdx.x, nth = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
@@ -643,8 +642,6 @@ __device__ __forceinline__ void cr_body(const CrArgs<C>& A, const SlabDev& sd, i
     const C* cf = A.coef + sd.coef_off;
     C* tg = tb + (size_t)(warp * GPW + grp) * G;
     auto row = [&](int k) { return b + (long long)k * lw; };
-    const long long nt2 = (long long)K * K;
-    constexpr bool kPart = MODE == CR_A;
     const CrChunk* tab = G == 16 ? A.tab16 : A.tab32;
     const int ntab = G == 16 ? A.n16 : A.n32;
 
@@ -671,35 +668,10 @@ __device__ __forceinline__ void cr_body(const CrArgs<C>& A, const SlabDev& sd, i
         for (int st = 0; st < A.nst; ++st) issue_next(st);
 
     // ---- right-hand side
-    for (int e = tid; e < NR * K * lw; e += nth) {   // right-hand side r + e / (K lw), block row k
-        const int pp = e % lw;
-        const int k = (e / lw) % K;
-        const int rq = r + e / (K * lw);
+    for (int e = tid; e < K * lw; e += nth) {
+        const int pp = e % lw, k = e / lw;
         C v = czero<C>();
-        if (pp < w && rq < A.R) {
-            const int r = rq;
-            if (MODE == CR_A || MODE == CR_E) {
-                if (pp >= na && pp <= sd.ll) v = A.f[(long long)r * nt2 + (long long)k * K + sd.s + A.b + (pp - na)];
-                if (MODE == CR_E) {
-                    const C* ck = cf + (long long)k * sd.cstride + pp * 9;
-                    const long long vec = (long long)K * A.R;
-                    if (pp == na && i > 0)
-                        for (int dk = -1; dk <= 1; ++dk) {
-                            const int kk = k + dk;
-                            if (kk >= 0 && kk < K)
-                                v = cfnma(ck[dk + 1], A.lam[(long long)(i - 1) * vec + (long long)kk * A.R + r], v);
-                        }
-                    if (pp == sd.ll && i < A.n_slabs - 1)
-                        for (int dk = -1; dk <= 1; ++dk) {
-                            const int kk = k + dk;
-                            if (kk >= 0 && kk < K)
-                                v = cfnma(ck[6 + dk + 1], A.phi[(long long)(i + 1) * vec + (long long)kk * A.R + r], v);
-                        }
-                }
-            } else {
-                if (pp >= na && pp <= sd.ll) v = to_c<C>(A.v_in[((long long)r * sd.nl + (pp - na)) * K + k]);
-            }
-        }
+        if (pp < w && pp >= na && pp <= sd.ll) v = to_c<C>(A.v_in[((long long)r * sd.nl + (pp - na)) * K + k]);
         b[e] = v;
     }
     __syncthreads();   // b written, first descriptors published
@@ -722,7 +694,7 @@ __device__ __forceinline__ void cr_body(const CrArgs<C>& A, const SlabDev& sd, i
         // products are split over four warps (column quarters, or block x half
         // of the columns in the two-block phases) and the partial sums meet in
         // shared memory after one more barrier
-        const bool split = cr_split_phase(G, kind, l, kPart);
+        const bool split = cr_split_phase(G, kind, l);
         if (split) {
             C* part = tb + kSolveThreads;   // kSplitRows x 4 x 32 partial sums
             for (int t0 = warp; t0 < cnt * 4; t0 += nw) {   // one warp per (row, part); G == 32
@@ -769,14 +741,9 @@ __device__ __forceinline__ void cr_body(const CrArgs<C>& A, const SlabDev& sd, i
                 x[p] = (kind == PH_FODD || kind == PH_TOP) ? sum : x[p] - sum;
             }
         } else
-        for (int t0 = warp * GPW; t0 < cnt * NR; t0 += nw * GPW) {
-            // task = (right-hand side q, row t of the chunk)
-            const int tq = t0 + grp;
-            const bool on = tq < cnt * NR;
-            const int q = on ? tq / cnt : 0;
-            const int t = on ? tq - q * cnt : 0;
-            C* const bq = b + (long long)q * K * lw;
-            auto row = [&](int k) { return bq + (long long)k * lw; };
+        for (int t0 = warp * GPW; t0 < cnt; t0 += nw * GPW) {
+            const bool on = t0 + grp < cnt;
+            const int t = on ? t0 + grp : 0;
             const int rr = r0 + t;
             C acc[CPT];
             if (kind == PH_FODD || kind == PH_TOP) {
@@ -825,67 +792,25 @@ __device__ __forceinline__ void cr_body(const CrArgs<C>& A, const SlabDev& sd, i
                 }
                 const C* Dp = S + (size_t)cnt * 6 * G;
                 C* x = row(k);
-                if (!kPart) {
-                    tg[p] = tv;
-                    __syncwarp();
-                    acc[0] = on ? x[p] : czero<C>();
-                    if (on) mv_cols<C, G, CPT, true>(Dp + (size_t)t * bs, p, tg, G, nc, acc);
-                    if (on) x[p] = acc[0];
-                    __syncwarp();
-                } else {
-                    // only layers na and ll: the two rows of D^{-1} against t, reduced over the group
-                    const C* pr = Dp + (size_t)t * 2 * G;
-                    const C q0 = on ? pr[p] : czero<C>(), q1 = on ? pr[G + p] : czero<C>();
-                    C d0 = q0 * tv, d1 = q1 * tv;
-#pragma unroll
-                    for (int off = G / 2; off > 0; off >>= 1) {
-                        d0.x += __shfl_xor_sync(0xffffffffu, d0.x, off, G);
-                        d0.y += __shfl_xor_sync(0xffffffffu, d0.y, off, G);
-                        d1.x += __shfl_xor_sync(0xffffffffu, d1.x, off, G);
-                        d1.y += __shfl_xor_sync(0xffffffffu, d1.y, off, G);
-                    }
-                    if (on && p == na) x[na] = x[na] - d0;
-                    if (on && p == sd.ll && sd.ll != na) x[sd.ll] = x[sd.ll] - d1;
-                }
+                tg[p] = tv;
+                __syncwarp();
+                acc[0] = on ? x[p] : czero<C>();
+                if (on) mv_cols<C, G, CPT, true>(Dp + (size_t)t * bs, p, tg, G, nc, acc);
+                if (on) x[p] = acc[0];
+                __syncwarp();
             }
         }
         __syncthreads();   // the stage is free, the phase's rows are written
         if (tid == 0) issue_next(g + A.nst);
     }
 
-    // ---- outputs, per right-hand side
-    for (int q = 0; q < NR; ++q) {
-        const int rq = r + q;
-        if (rq >= A.R) break;
-        C* const bq = b + (long long)q * K * lw;
-        auto rowo = [&](int k) { return bq + (long long)k * lw; };
-        if (MODE == CR_A) {
-            const long long base = (long long)i * K * A.R + rq;
-            for (int k = tid; k < K; k += nth) {
-                A.a_first[base + (long long)k * A.R] = rowo(k)[na];
-                A.a_last[base + (long long)k * A.R] = rowo(k)[sd.ll];
-            }
-        } else if (MODE == CR_E) {
-            const int nl = sd.nl;
-            for (int e = tid; e < nl * K; e += nth) {
-                const int k = e % K, pp = na + e / K;
-                const int x1 = sd.s + (pp - na), i2 = k - A.b;
-                if (A.y_grid)
-                    A.y[(long long)rq * A.n_tot * A.n_tot + (long long)k * A.n_tot + (x1 + A.b)] = to_d(rowo(k)[pp]);
-                else if (x1 >= 1 && x1 <= A.n && i2 >= 1 && i2 <= A.n)
-                    A.y[(long long)rq * A.n * A.n + (long long)(x1 - 1) * A.n + (i2 - 1)] = to_d(rowo(k)[pp]);
-            }
-        } else {
-            const int nl = sd.nl;
-            for (int e = tid; e < nl * K; e += nth) {
-                const int k = e % K, pp = na + e / K;
-                A.w_out[((long long)rq * nl + (pp - na)) * K + k] = to_d(rowo(k)[pp]);
-            }
-        }
+    for (int e = tid; e < sd.nl * K; e += nth) {
+        const int k = e % K, pp = na + e / K;
+        A.w_out[((long long)r * sd.nl + (pp - na)) * K + k] = to_d(row(k)[pp]);
     }
 }
 
-template <typename T, int MODE, int NR = 1>
+template <typename T>
 __global__ void __launch_bounds__(kSolveThreads) cr_solve_kernel(CrArgs<cx<T>> A) {
     using C = cx<T>;
     __shared__ CrLv lv[33];
@@ -906,16 +831,10 @@ __global__ void __launch_bounds__(kSolveThreads) cr_solve_kernel(CrArgs<cx<T>> A
     }
     bool ok = true;
     __syncthreads();
-    int i, r;
-    long long cta;
-    if (MODE == CR_TEST) { i = A.slab; r = blockIdx.x; cta = blockIdx.x; }
-    // slab-major grid: a slab's right-hand sides run together and share its factor stream in L2
-    else { i = A.slab0 + blockIdx.y; r = blockIdx.x * NR; cta = (long long)blockIdx.y * gridDim.x + blockIdx.x; }
-    const SlabDev sd = A.slabs[i];
-    C* b = A.bsm ? reinterpret_cast<C*>(sms) : A.bg + cta * A.bstride;
-    if (sd.w <= 16) cr_body<C, MODE, 16, NR>(A, sd, i, r, b, tb, ring, full, desc, lv, ok);
-    else if constexpr (NR == 1) cr_body<C, MODE, 32, 1>(A, sd, i, r, b, tb, ring, full, desc, lv, ok);
-    else if (threadIdx.x == 0) atomicOr(A.err, LSS_DERR_CONFIG);   // the host launches NR > 1 for 16-wide slabs only
+    const SlabDev sd = A.slabs[A.slab];
+    C* b = A.bsm ? reinterpret_cast<C*>(sms) : A.bg + (long long)blockIdx.x * A.bstride;
+    if (sd.w <= 16) cr_body<C, 16>(A, sd, A.slab, blockIdx.x, b, tb, ring, full, desc, lv, ok);
+    else cr_body<C, 32>(A, sd, A.slab, blockIdx.x, b, tb, ring, full, desc, lv, ok);
     if (__syncthreads_or(!ok) && threadIdx.x == 0) {
         // a wait expired: give the copies already issued a bounded chance to land
         const long long t0 = clock64();
@@ -1460,27 +1379,18 @@ struct SolvePlan {
     int bsm, nst, stage_ent;
     size_t sh;
 };
-// ldw > 0: plan for slabs of that block width only.
 template <typename C>
-bool plan_solve(const lss_ctx* c, size_t bb, size_t tb, bool allow_smem_b, SolvePlan* P, int ldw = 0) {
-    const long long row_ent = ldw > 0 ? std::max<long long>(2LL * ldw * ldw, 6LL * ldw + (long long)ldw * ldw)
-                                      : max_row_ent(c);
+bool plan_solve(const lss_ctx* c, size_t bb, size_t tb, bool allow_smem_b, SolvePlan* P) {
+    const long long row_ent = max_row_ent(c);
     const size_t min_stage = sizeof(C) * (size_t)row_ent;
     const size_t want = std::max<size_t>(48 * 1024, min_stage);
-    if (c->tune.solve_bsm == 0) allow_smem_b = false;
-    const int tn = (ldw == 32 && c->tune.solve_nst_w) ? c->tune.solve_nst_w : c->tune.solve_nst;
-    // half the budget leaves room for a second CTA on the SM (latency hiding)
-    const size_t budget = c->tune.solve_half ? kSmemBudget / 2 : kSmemBudget;
     for (int bsm = allow_smem_b ? 1 : 0; bsm >= 0; --bsm) {
         const size_t fixed = tb + (bsm ? bb : 0);
-        if (fixed + 2 * min_stage > budget) continue;
-        const size_t avail = budget - fixed;
+        if (fixed + 2 * min_stage > kSmemBudget) continue;
+        const size_t avail = kSmemBudget - fixed;
         int nst = (int)std::min<size_t>(4, avail / want);
         size_t stage = want;
-        if (tn >= 2 && avail / tn >= min_stage) {   // tuned: tn stages sharing the free shared memory
-            nst = tn;
-            stage = (avail / tn) / 16 * 16;
-        } else if (nst < 2) {
+        if (nst < 2) {
             nst = 2;
             stage = (avail / 2) / 16 * 16;
         }
@@ -1493,21 +1403,21 @@ bool plan_solve(const lss_ctx* c, size_t bb, size_t tb, bool allow_smem_b, Solve
     return false;
 }
 
-// Chunk tables (16- and 32-wide blocks) of one output kind and stage size,
+// Chunk tables (16- and 32-wide blocks) of one stage size,
 // built and uploaded on first use (on stream s, ahead of the solves that read
 // them: a copy on the legacy default stream would not be ordered before
 // kernels on a non-blocking stream).
-int chunk_tables(lss_ctx* c, bool part, int stage_ent, CrArgsTables* out, cudaStream_t s) {
+int chunk_tables(lss_ctx* c, int stage_ent, CrArgsTables* out, cudaStream_t s) {
     for (size_t q = 0; q < c->chunk_keys.size(); ++q)
-        if (c->chunk_keys[q][0] == (part ? 1 : 0) && c->chunk_keys[q][1] == stage_ent) {
+        if (c->chunk_keys[q][0] == stage_ent) {
             out->t16 = c->chunk_dev[2 * q];
             out->t32 = c->chunk_dev[2 * q + 1];
-            out->n16 = (int)c->chunk_keys[q][2];
-            out->n32 = (int)c->chunk_keys[q][3];
+            out->n16 = (int)c->chunk_keys[q][1];
+            out->n32 = (int)c->chunk_keys[q][2];
             return LSS_OK;
         }
-    const std::vector<CrChunk> t16 = cr_chunk_table(c->n_tot, 16, part, stage_ent, kSolveThreads / 16);
-    const std::vector<CrChunk> t32 = cr_chunk_table(c->n_tot, 32, part, stage_ent, kSolveThreads / 32);
+    const std::vector<CrChunk> t16 = cr_chunk_table(c->n_tot, 16, stage_ent, kSolveThreads / 16);
+    const std::vector<CrChunk> t32 = cr_chunk_table(c->n_tot, 32, stage_ent, kSolveThreads / 32);
     void* d16 = nullptr;
     void* d32 = nullptr;
     cudaError_t e = cudaMalloc(&d16, t16.size() * sizeof(CrChunk));
@@ -1520,7 +1430,7 @@ int chunk_tables(lss_ctx* c, bool part, int stage_ent, CrArgsTables* out, cudaSt
         if (d32) cudaFree(d32);
         return lss_check_cuda(c, e, "chunk tables");
     }
-    c->chunk_keys.push_back({part ? 1LL : 0LL, (long long)stage_ent, (long long)t16.size(), (long long)t32.size()});
+    c->chunk_keys.push_back({(long long)stage_ent, (long long)t16.size(), (long long)t32.size()});
     c->chunk_dev.push_back(d16);
     c->chunk_dev.push_back(d32);
     out->t16 = d16;
@@ -1534,25 +1444,22 @@ int chunk_tables(lss_ctx* c, bool part, int stage_ent, CrArgsTables* out, cudaSt
 // sides per CTA: in shared memory when they fit (and no fixed scratch is
 // given), else in global scratch (the fixed array `scratch`, or the context's
 // growable buffer).
-// ldw > 0: the launch covers slabs of that block width only (its right-hand
-// sides and stages are sized for it); z_off: byte offset of this launch's part
-// of the context's global right-hand-side scratch.
-template <typename T, int MODE, int NR = 1>
+template <typename T>
 int launch_solve(lss_ctx* c, CrArgs<cx<T>> A, dim3 grid, long long per_cta, void* scratch, size_t scratch_bytes,
-                 cudaStream_t s, int ldw = 0, size_t z_off = 0) {
+                 cudaStream_t s) {
     using C = cx<T>;
-    auto kern = cr_solve_kernel<T, MODE, NR>;
+    auto kern = cr_solve_kernel<T>;
     const size_t tb = sizeof(C) * ((size_t)kSolveThreads + kSplitRows * 4 * 32);
     const size_t bb = sizeof(C) * (size_t)per_cta;
     SolvePlan P;
-    if (!plan_solve<C>(c, bb, tb, scratch == nullptr, &P, ldw))
+    if (!plan_solve<C>(c, bb, tb, scratch == nullptr, &P))
         return lss_fail(c, LSS_ERR_UNSUPPORTED, "slab solve: the factor stream does not fit in shared memory");
     A.bstride = per_cta;
     A.bsm = P.bsm;
     A.nst = P.nst;
     A.stage_ent = P.stage_ent;
     CrArgsTables tabs;
-    int rc = chunk_tables(c, MODE == CR_A, P.stage_ent, &tabs, s);
+    int rc = chunk_tables(c, P.stage_ent, &tabs, s);
     if (rc) return rc;
     A.tab16 = (const CrChunk*)tabs.t16;
     A.tab32 = (const CrChunk*)tabs.t32;
@@ -1569,10 +1476,10 @@ int launch_solve(lss_ctx* c, CrArgs<cx<T>> A, dim3 grid, long long per_cta, void
                                     " bytes of scratch, the fixed scratch holds " + std::to_string(scratch_bytes) +
                                     " (use fewer right-hand sides per call)");
             A.bg = (C*)scratch;
-        } else {   // z_off: this launch's part of a scratch shared by concurrent launches
-            rc = lss_grow(c, &c->z_buf, &c->z_cap, z_off + need);
+        } else {
+            rc = lss_grow(c, &c->z_buf, &c->z_cap, need);
             if (rc) return rc;
-            A.bg = (C*)((char*)c->z_buf + z_off);
+            A.bg = (C*)c->z_buf;
         }
     }
     kern<<<grid, kSolveThreads, P.sh, s>>>(A);
@@ -2037,25 +1944,22 @@ int prepare_chunk_tables(lss_ctx* c, cudaStream_t s) {
         SolvePlan P;
         if (plan_solve<C>(c, bb, tb, smem_b == 1, &P)) plans.push_back(P);
     }
-    for (const SweepRun& u : sweep_runs(c)) {
-        SolvePlan P;
-        for (int nr = 1; nr <= (u.ldw == 16 ? 2 : 1); ++nr)   // one or two right-hand sides per CTA
-            for (int smem_b = 0; smem_b < 2; ++smem_b)
-                if (plan_solve<C>(c, sizeof(C) * (size_t)nr * c->n_tot * u.ldw, tb, smem_b == 1, &P, u.ldw))
-                    plans.push_back(P);
+    for (const SolvePlan& P : plans) {
+        CrArgsTables t;
+        const int rc = chunk_tables(c, P.stage_ent, &t, s);
+        if (rc) return rc;
     }
-    for (const SolvePlan& P : plans)
-        for (int part = 0; part < 2; ++part) {
-            CrArgsTables t;
-            const int rc = chunk_tables(c, part == 1, P.stage_ent, &t, s);
-            if (rc) return rc;
-        }
     return LSS_OK;
 }
 
-// One sweep pass (MODE CR_A or CR_E) over every slab, run by run.
-// Block LU solves switched off by LSS_SLAB_SOLVE=cr (cyclic reduction for every run).
-bool thomas_enabled() {
+// The block LU's right-hand sides share a chain of 2 n_tot block rows per CTA,
+// which pays where the arithmetic is cheap: in double precision 65 x 1 CTAs
+// (n = 256, 16 right-hand sides) took 14 ms per pass, bound by the FP64 pipe
+// of 65 SMs, the cluster solves (cr_cluster.cu) 2.9.  In single precision at
+// n = 512 with 64 it takes 4.1 ms per pass where they take 5.5.
+// LSS_SLAB_SOLVE=cr: cyclic reduction for every run.
+bool thomas_enabled(const lss_ctx* c) {
+    if (c->prec == LSS_FP64) return false;
     const char* v = std::getenv("LSS_SLAB_SOLVE");
     return !(v && v[0] == 'c');
 }
@@ -2110,12 +2014,13 @@ size_t thomas_scratch(const lss_ctx* c, int nsl, int R) {
     return sizeof(cx<T>) * (size_t)((R + nrb - 1) / nrb) * nsl * c->n_tot * 16 * nrb;
 }
 
+// The 16-wide runs go to the block LU when the caller prepared its factors,
+// everything else to the cyclic reduction on clusters.
 template <typename T, int MODE>
 int sweep_pass(lss_ctx* c, CrArgs<cx<T>> A, int R, cudaStream_t s, bool thomas = false) {
     const std::vector<SweepRun> runs = sweep_runs(c);
     int rc = lss_ensure_aux(c, runs.size());
     if (rc) return rc;
-    // 16-wide runs by the block LU when the caller prepared its factors
     auto th_run = [&](const SweepRun& u) { return thomas && u.ldw == 16; };
     size_t qtot = 0;
     std::vector<size_t> qoff(runs.size());
@@ -2124,33 +2029,29 @@ int sweep_pass(lss_ctx* c, CrArgs<cx<T>> A, int R, cudaStream_t s, bool thomas =
         if (th_run(runs[ri])) qtot += thomas_scratch<T>(c, runs[ri].n, R);
     }
     if (qtot && (rc = lss_grow(c, &c->tq_buf, &c->tq_cap, qtot))) return rc;
-    // global right-hand-side scratch of every run, grown before any launch so
-    // that concurrent runs use disjoint parts of one buffer
-    // right-hand sides per CTA: two on 16-wide runs when the autotuner chose so
-    auto nr_of = [&](const SweepRun& u) { return (c->tune.solve_nr == 2 && u.ldw == 16 && R >= 2) ? 2 : 1; };
-    size_t ztot = 0;
-    std::vector<size_t> zoff(runs.size());
-    for (size_t ri = 0; ri < runs.size(); ++ri) {
-        const int nr = nr_of(runs[ri]);
-        zoff[ri] = ztot;
-        ztot += sizeof(cx<T>) * (size_t)c->n_tot * runs[ri].ldw * nr * ((R + nr - 1) / nr) * runs[ri].n;
-    }
-    if ((rc = lss_grow(c, &c->z_buf, &c->z_cap, ztot))) return rc;
+    CrcArgs Q{};
+    Q.R = R;
+    Q.f = A.f;
+    Q.a_first = A.a_first;
+    Q.a_last = A.a_last;
+    Q.lam = A.lam;
+    Q.phi = A.phi;
+    Q.y = A.y;
+    Q.y_grid = A.y_grid;
     if (runs.size() > 1) cudaEventRecord(c->fork_event, s);
     for (size_t ri = 0; ri < runs.size() && !rc; ++ri) {
         const SweepRun& u = runs[ri];
         cudaStream_t su = ri == 0 ? s : c->aux_stream[ri - 1];
         if (ri > 0) cudaStreamWaitEvent(su, c->fork_event, 0);
-        CrArgs<cx<T>> Ar = A;
-        Ar.slab0 = u.s0;
-        if (th_run(u))
-            rc = launch_thomas<T, MODE>(c, Ar, u.n, R, su, qoff[ri]);
-        else if (nr_of(u) == 2)
-            rc = launch_solve<T, MODE, 2>(c, Ar, dim3((R + 1) / 2, u.n), 2LL * c->n_tot * u.ldw, nullptr, 0, su, u.ldw,
-                                          zoff[ri]);
-        else
-            rc = launch_solve<T, MODE>(c, Ar, dim3(R, u.n), (long long)c->n_tot * u.ldw, nullptr, 0, su, u.ldw,
-                                       zoff[ri]);
+        if (th_run(u)) {
+            if constexpr (sizeof(T) == 4) {
+                CrArgs<cx<T>> Ar = A;
+                Ar.slab0 = u.s0;
+                rc = launch_thomas<T, MODE>(c, Ar, u.n, R, su, qoff[ri]);
+            }
+        } else {
+            rc = lss_cr_cluster(c, MODE == CR_A ? CRC_A : CRC_E, false, Q, u.s0, u.n, u.ldw, su);
+        }
         if (ri > 0) {
             cudaEventRecord(c->aux_event[ri - 1], su);
             cudaStreamWaitEvent(s, c->aux_event[ri - 1], 0);
@@ -2187,13 +2088,14 @@ int factor_impl(lss_ctx* c, cudaStream_t s) {
     if ((rc = lss_ensure_aux(c, runs.size() + 1))) return rc;
     // the block LU factors (when this context's sweeps use them) on the last
     // auxiliary stream, joined at the end of the factorization
-    const bool chain = c->th_wanted && thomas_enabled();
+    const bool chain = c->th_wanted && thomas_enabled(c);
     cudaStream_t sch = c->aux_stream[runs.size() - 1];
     if (chain) {
         if ((rc = lss_grow(c, &c->th_buf, &c->th_cap, sizeof(C) * (size_t)ns * 3 * K0 * 256))) return rc;
         cudaEventRecord(c->fork_event, s);
         cudaStreamWaitEvent(sch, c->fork_event, 0);
-        th_chain_kernel<T><<<ns, 32, 0, sch>>>(c->d_slabs, (const C*)c->coef, (C*)c->th_buf, K0, c->d_err);
+        if constexpr (sizeof(T) == 4)
+            th_chain_kernel<T><<<ns, 32, 0, sch>>>(c->d_slabs, (const C*)c->coef, (C*)c->th_buf, K0, c->d_err);
         if ((rc = lss_check_cuda(c, cudaGetLastError(), "block LU factorization launch"))) return rc;
     }
     {
@@ -2525,12 +2427,12 @@ int sweep_impl(lss_ctx* c, const double2* r, double2* y, int R, cudaStream_t s, 
     // block LU solves for the 16-wide slabs with many right-hand sides; their
     // factors are computed here when missing, but never inside a stream
     // capture (a captured sweep without them uses the cyclic reduction)
-    bool thomas = R >= kThMinR && thomas_enabled();
+    bool thomas = R >= kThMinR && thomas_enabled(c);
     if (thomas && !c->th_valid) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         cudaStreamIsCapturing(s, &cap);
         if (cap != cudaStreamCaptureStatusNone) thomas = false;
-        else if ((rc = thomas_prepare_t<T>(c, s))) return rc;
+        else if ((rc = thomas_prepare_t<float>(c, s))) return rc;
     }
     if (c->n_slabs > 1) {
         {
@@ -2555,9 +2457,9 @@ int slab_apply_impl(lss_ctx* c, int slab, const double2* v, double2* w, int R, v
     A.v_in = v;
     A.w_out = w;
     const long long per_cta = (long long)c->n_tot * ldwmax_of(c);
-    if (scratch) return launch_solve<T, CR_TEST>(c, A, dim3(R), per_cta, scratch, scratch_bytes, s);
+    if (scratch) return launch_solve<T>(c, A, dim3(R), per_cta, scratch, scratch_bytes, s);
     ProfScope ps(c, s, LSS_PROF_SLAB_E, 1);
-    return launch_solve<T, CR_TEST>(c, A, dim3(R), per_cta, nullptr, 0, s);
+    return launch_solve<T>(c, A, dim3(R), per_cta, nullptr, 0, s);
 }
 
 }  // namespace
@@ -2582,12 +2484,8 @@ int lss_ensure_aux(lss_ctx* c, size_t n) {
 }
 
 int lss_thomas_prepare(lss_ctx* c, int R, cudaStream_t s) {
-    if (c->dim != 2 || R < kThMinR || !thomas_enabled() || c->th_valid) return LSS_OK;
-    return c->prec == LSS_FP64 ? thomas_prepare_t<double>(c, s) : thomas_prepare_t<float>(c, s);
-}
-
-int lss_prepare_solve_tables(lss_ctx* c, cudaStream_t s) {
-    return c->prec == LSS_FP64 ? prepare_chunk_tables<double>(c, s) : prepare_chunk_tables<float>(c, s);
+    if (c->dim != 2 || R < kThMinR || !thomas_enabled(c) || c->th_valid) return LSS_OK;
+    return thomas_prepare_t<float>(c, s);
 }
 
 int lss_factor_slabs(lss_ctx* c, cudaStream_t s) {

@@ -1,8 +1,7 @@
 // Autotuner: times the context's own operations with CUDA events for each
 // admissible value of the launch parameters that do not change any result
-// (which columns share an FFT CTA, how the slab-solve factor ring divides
-// shared memory and whether the right-hand sides stay in it, how many map
-// stages the recurrence keeps in flight) and keeps the fastest.  Every
+// (which columns share an FFT CTA, how many map stages the recurrence keeps in
+// flight) and keeps the fastest.  Every
 // candidate computes each output with the same arithmetic in the same order,
 // so tuned and untuned solves agree bit for bit.
 #include <algorithm>
@@ -70,41 +69,8 @@ int tune_one(lss_ctx* c, int R, cudaStream_t s) {
         }
         c->tune.fft_C = pick ? pick : keep.fft_C;
     }
-    // slab-solve plan, then the recurrence ring: one preconditioner apply
+    // the recurrence ring: one preconditioner apply
     auto sweep = [&] { return lss_sweep(c, x, y, R, s); };
-    {
-        float best = -1;
-        lss_ctx::Tune pick = c->tune;
-        for (int nr : {1, 2})
-            for (int half : {0, 1})
-                for (int bsm : {-1, 0})
-                    for (int nst : {0, 2, 3, 4}) {
-                        if (nr == 2 && (R < 2 || half)) continue;   // two right-hand sides need the whole budget
-                        c->tune.solve_nr = nr;
-                        c->tune.solve_half = half;
-                        c->tune.solve_bsm = bsm;
-                        c->tune.solve_nst = nst;
-                        const float ms = time_ms(t, s, 3, sweep);
-                        if (ms > 0 && (best < 0 || ms < best)) { best = ms; pick = c->tune; }
-                    }
-        c->tune = pick;
-    }
-    {   // ring stages of the 32-wide slabs' own launches (they set each pass's critical path)
-        bool wide = false;
-        for (const auto& sd : c->slabs) wide |= sd.ldw == 32;
-        bool narrow = false;
-        for (const auto& sd : c->slabs) narrow |= sd.ldw == 16;
-        if (wide && narrow) {
-            float best = -1;
-            int pick = 0;
-            for (int nst : {0, 2, 3, 4}) {
-                c->tune.solve_nst_w = nst;
-                const float ms = time_ms(t, s, 3, sweep);
-                if (ms > 0 && (best < 0 || ms < best)) { best = ms; pick = nst; }
-            }
-            c->tune.solve_nst_w = pick;
-        }
-    }
     {
         float best = -1;
         int pick = c->tune.rec_nb;
@@ -121,10 +87,7 @@ int tune_one(lss_ctx* c, int R, cudaStream_t s) {
     cudaGetLastError();   // a refused candidate leaves no error behind
     c->err = err0;
     ++c->buf_gen;         // captured iterations used the old launch parameters
-    // tables of every plan the entry points may now use (the fixed-scratch
-    // slab operator must not build one later)
-    int rc = lss_prepare_solve_tables(c, s);
-    if (!rc) rc = lss_check_device_err(c, s);
+    int rc = lss_check_device_err(c, s);
     return rc;
 }
 
@@ -147,12 +110,12 @@ extern "C" int lss_autotune(lss_ctx* c, int R, int* chosen, void* stream) {
     if (chosen) {
         const lss_ctx::Tune& t = c->inst.empty() ? c->tune : c->inst[0]->tune;
         chosen[0] = t.fft_C;
-        chosen[1] = t.solve_bsm;
-        chosen[2] = t.solve_nst;
+        chosen[1] = -1;   // the slab solves size themselves (cr_cluster.cu)
+        chosen[2] = 0;
         chosen[3] = t.rec_nb;
-        chosen[4] = t.solve_nst_w;
-        chosen[5] = t.solve_half;
-        chosen[6] = t.solve_nr;
+        chosen[4] = 0;
+        chosen[5] = 0;
+        chosen[6] = 1;
     }
     return LSS_OK;
 }
