@@ -85,10 +85,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Persistent: CTA loops over (slab, row tile, column tile) slots.  128 threads.
-__global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ slabs, int n_slabs,
+// Persistent: CTA loops over the tiles of every slab in turn.  A tile is a
+// chain of loads, products and a read-modify-write of W, so what bounds it is
+// the warps that share an SM's latencies: 256 threads, of which one half stages
+// A while the other stages B, and the halves take alternate column chunks of
+// the epilogue.  (M = 984 .. 1476, 17 slabs: 120 us per launch with 128 threads
+// and the tile table of the widest slab, half of it empty, dealt round-robin.)
+constexpr int kTcThreads = 256;
+__global__ void __launch_bounds__(kTcThreads, 2) f3_update_tc(const Slab3* __restrict__ slabs, int n_slabs,
                                                      float2* __restrict__ W, const float2* __restrict__ T64, int J0,
-                                                     int NO, int Tld, int tmax, int* err) {
+                                                     int NO, int Tld, int* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char* Abig = sm;
     unsigned char* Asml = sm + kABytes;
@@ -97,6 +103,7 @@ __global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ sl
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + 2 * kABytes + 2 * kBBytes);
     uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + 2 * kABytes + 2 * kBBytes + 16);
     const int tid = threadIdx.x, warp = tid >> 5;
+    const int half = tid >> 7, t128 = tid & 127;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
@@ -115,16 +122,17 @@ __global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ sl
     unsigned phase = 0;
     bool ok = true;
 
-    const long long slots = (long long)n_slabs * tmax * tmax;
-    for (long long slot = blockIdx.x; slot < slots && ok; slot += gridDim.x) {
-        const int slab = (int)(slot / ((long long)tmax * tmax));
-        const int rem = (int)(slot % ((long long)tmax * tmax));
+    for (int slot = blockIdx.x, slab = 0, first = 0; ok; slot += gridDim.x) {
+        int tiles = 0;   // slab and tile of this slot (slabs already finished hold no tiles)
+        for (; slab < n_slabs; ++slab) {
+            tiles = J0 < slabs[slab].M ? (slabs[slab].M + 127) / 128 : 0;
+            if (slot < first + tiles * tiles) break;
+            first += tiles * tiles;
+        }
+        if (slab == n_slabs) break;
         const Slab3 sd = slabs[slab];
         const int M = sd.M;
-        if (J0 >= M) continue;
-        const int tiles = (M + 127) / 128;
-        const int ti = rem / tmax, tj = rem % tmax;
-        if (ti >= tiles || tj >= tiles) continue;
+        const int ti = (slot - first) / tiles, tj = (slot - first) % tiles;
         const int nbo = min(NO, M - J0);
         const int i0 = ti * 128, c0 = tj * 128;
         float2* w = W + sd.w_off;
@@ -135,8 +143,8 @@ __global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ sl
         const float2* t = t64 + (long long)kc * kTcNB * Tld;
 
         // ---- operands into shared memory
-        {   // A: row tid of the tile, panel columns j0.. (2 nbp reals, zero beyond)
-            const int i = i0 + tid;
+        if (half == 0) {   // A: row t128 of the tile, panel columns j0.. (2 nbp reals, zero beyond)
+            const int i = i0 + t128;
             float a[kTcK];
             for (int q = 0; q < kTcNB; ++q) {
                 float2 v = make_float2(0.f, 0.f);
@@ -150,12 +158,12 @@ __global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ sl
                 split_tf32(a[4 * k4 + 1], hb.y, hs.y);
                 split_tf32(a[4 * k4 + 2], hb.z, hs.z);
                 split_tf32(a[4 * k4 + 3], hb.w, hs.w);
-                *reinterpret_cast<float4*>(Abig + core_off(tid, 4 * k4)) = hb;
-                *reinterpret_cast<float4*>(Asml + core_off(tid, 4 * k4)) = hs;
+                *reinterpret_cast<float4*>(Abig + core_off(t128, 4 * k4)) = hb;
+                *reinterpret_cast<float4*>(Asml + core_off(t128, 4 * k4)) = hs;
             }
         }
-        {   // B^T rows 2c, 2c+1 for complex column c = tid: K entries (2kk, 2kk+1)
-            const int c = c0 + tid;
+        else {   // B^T rows 2c, 2c+1 for complex column c = t128: K entries (2kk, 2kk+1)
+            const int c = c0 + t128;
             float r0[kTcK], r1[kTcK];
             for (int q = 0; q < kTcNB; ++q) {
                 float2 v = make_float2(0.f, 0.f);
@@ -175,10 +183,10 @@ __global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ sl
                 split_tf32(r1[4 * k4 + 1], b1.y, s1.y);
                 split_tf32(r1[4 * k4 + 2], b1.z, s1.z);
                 split_tf32(r1[4 * k4 + 3], b1.w, s1.w);
-                *reinterpret_cast<float4*>(Bbig + core_off(2 * tid, 4 * k4)) = b0;
-                *reinterpret_cast<float4*>(Bsml + core_off(2 * tid, 4 * k4)) = s0;
-                *reinterpret_cast<float4*>(Bbig + core_off(2 * tid + 1, 4 * k4)) = b1;
-                *reinterpret_cast<float4*>(Bsml + core_off(2 * tid + 1, 4 * k4)) = s1;
+                *reinterpret_cast<float4*>(Bbig + core_off(2 * t128, 4 * k4)) = b0;
+                *reinterpret_cast<float4*>(Bsml + core_off(2 * t128, 4 * k4)) = s0;
+                *reinterpret_cast<float4*>(Bbig + core_off(2 * t128 + 1, 4 * k4)) = b1;
+                *reinterpret_cast<float4*>(Bsml + core_off(2 * t128 + 1, 4 * k4)) = s1;
             }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -212,31 +220,31 @@ __global__ void __launch_bounds__(128) f3_update_tc(const Slab3* __restrict__ sl
 
         // ---- epilogue, 8 chunks of 16 complex columns: each thread moves its
         // accumulator row (tcgen05.ld) into shared memory (row stride 33
-        // floats, no bank conflicts), then the CTA adds the chunk to W with
-        // consecutive threads on consecutive columns of a row
-        float* S = reinterpret_cast<float*>(sm);   // the operands are consumed
-        for (int ch = 0; ch < kTileN / 32; ++ch) {
+        // floats, no bank conflicts), then its half of the CTA adds the chunk
+        // to W with consecutive threads on consecutive columns of a row
+        float* S = reinterpret_cast<float*>(sm) + half * 128 * 33;   // the operands are consumed
+        for (int ch = half; ch < kTileN / 32; ch += 2) {
             float v[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(ch * 32), v);
+            tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(ch * 32), v);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) S[tid * 33 + j] = v[j];
-            __syncthreads();
+            for (int j = 0; j < 32; ++j) S[t128 * 33 + j] = v[j];
+            asm volatile("bar.sync %0, 128;" ::"r"(half + 1) : "memory");
             float2 o[16];   // 16 independent loads, then the adds and stores
 #pragma unroll
             for (int u = 0; u < 16; ++u) {
-                const int e = tid + u * 128, row = e >> 4, q = e & 15;
+                const int e = t128 + u * 128, row = e >> 4, q = e & 15;
                 const int i = i0 + row, c = c0 + ch * 16 + q;
                 const bool ok_ = i < M && c < M && !(c >= J0 && c < J0 + nbo);
                 o[u] = ok_ ? w[(long long)i * M + c] : make_float2(0.f, 0.f);
             }
 #pragma unroll
             for (int u = 0; u < 16; ++u) {
-                const int e = tid + u * 128, row = e >> 4, q = e & 15;
+                const int e = t128 + u * 128, row = e >> 4, q = e & 15;
                 const int i = i0 + row, c = c0 + ch * 16 + q;
                 if (i >= M || c >= M || (c >= J0 && c < J0 + nbo)) continue;
                 w[(long long)i * M + c] = make_float2(o[u].x + S[row * 33 + 2 * q], o[u].y + S[row * 33 + 2 * q + 1]);
             }
-            __syncthreads();
+            asm volatile("bar.sync %0, 128;" ::"r"(half + 1) : "memory");
         }
         // the next tile's operand writes must not overtake this tile's reads
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -269,10 +277,11 @@ int lss3_update_tc(lss_ctx* c, float2* W, const float2* T64, int J0, int NO, cud
             done = 1;
         }
     }
-    const int tmax = (d->Mmax + 127) / 128;
-    const long long slots = (long long)c->n_slabs * tmax * tmax;
-    const int grid = (int)std::min<long long>(slots, 2LL * c->num_sms);
-    f3_update_tc<<<grid, 128, kTcSmem, s>>>(d->d_slabs, c->n_slabs, W, T64, J0, NO, d->Mmax, tmax, c->d_err);
+    int tiles = 0;
+    for (const Slab3& sd : d->slabs)
+        if (J0 < sd.M) tiles += ((sd.M + 127) / 128) * ((sd.M + 127) / 128);
+    const int grid = std::max(1, std::min(tiles, 2 * c->num_sms));
+    f3_update_tc<<<grid, kTcThreads, kTcSmem, s>>>(d->d_slabs, c->n_slabs, W, T64, J0, NO, d->Mmax, c->d_err);
     return lss_check_cuda(c, cudaGetLastError(), "tensor-core update launch");
 }
 
