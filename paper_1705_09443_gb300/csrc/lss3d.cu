@@ -24,6 +24,8 @@
 
 #include "fft_line.cuh"
 #include "fx_fft.cuh"
+#include <cooperative_groups.h>
+
 #include "lss_common.cuh"
 #include "lss_ctx.h"
 #include "lss3d.h"
@@ -33,7 +35,7 @@ using cd = std::complex<double>;
 
 namespace {
 
-constexpr int kMaxBlock3 = 1760;      // largest pivot block M = w * n_tot (panel kernel shared memory: M x 128 B)
+constexpr int kMaxBlock3 = 1760;      // largest pivot block M = w * n_tot (panel kernel: a row per thread of four CTAs)
 constexpr int kNB64 = 8;              // Gauss-Jordan panel width, FP64
 constexpr int kNB32 = 16;             // Gauss-Jordan panel width, FP32
 constexpr int kNO = 64;               // outer panel width of the tensor-core path
@@ -472,154 +474,214 @@ __global__ void f3_rowid_init(const Slab3* __restrict__ slabs, int* __restrict__
         rowid[(long long)s * Mmax + r] = r;
 }
 
-// Gauss-Jordan elimination of the panel columns J = [j0, j0+nbp) of W (one CTA
-// per slab, the M x NB panel in shared memory, column-major so that the
-// threads of a warp, which own consecutive rows, touch consecutive words).  Pivot j = j0 + jj is the
-// largest |W[r][j]| over rows r >= j (ties to the lower row); rows j and r are
-// swapped inside the panel (the rest of the rows later, by f3_swap_extract),
-// recorded in piv and in rowid.  After the panel the columns J hold the
-// eliminated values: rows R = [j0, j0+nbp) the inverse E of the pivot block,
-// the other rows -P_O E.
+// The largest key of a warp and the lowest row that has it, in every lane.
+__device__ __forceinline__ void warp_pivot(float& v, int& row) {
+    const unsigned u = __float_as_uint(v), m = __reduce_max_sync(0xffffffffu, u);   // v >= 0: ordered as integers
+    row = (int)__reduce_min_sync(0xffffffffu, u == m ? (unsigned)row : 0x7fffffffu);
+    v = __uint_as_float(m);
+}
+__device__ __forceinline__ void warp_pivot(double& v, int& row) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, row, o);
+        if (ov > v || (ov == v && oi < row)) { v = ov; row = oi; }
+    }
+}
+
+// Gauss-Jordan elimination of the panel columns J = [j0, j0+nbp) of W (one
+// cluster per slab).  Pivot j = j0 + jj is the largest |W[r][j]| over rows r >= j
+// (ties to the lower row); rows j and r are swapped inside the panel (the rest
+// of the rows later, by f3_swap_extract), recorded in piv and in rowid.  After
+// the panel the columns J hold the eliminated values: rows R = [j0, j0+nbp) the
+// inverse E of the pivot block, the other rows -P_O E.
+// A pivot is a chain: the largest entry, its reciprocal, one update of the
+// panel.  The rows are split over the CTAs of a cluster, one row per thread in
+// registers; each CTA sends its candidate row (with the reciprocal of its
+// pivot) and the owner of row j that row to every CTA's shared memory, and one
+// cluster barrier later each picks the pivot itself.  The columns move down by
+// one register per pivot (the pivot column is always register 0), which keeps
+// the loop rolled.  Rows reach the registers through a swizzled tile, so that W
+// is read and written in whole segments.
+// M = 984 .. 1476, 16 columns, FP32: 30 us (67 with the panel of a slab in one
+// CTA's shared memory, 52 in one CTA's registers, which spill at three rows per
+// thread; unrolled over the pivots 80, bound by the instruction fetch).
+constexpr int kPanelThreads = 448, kPanelCtas = 4;
+static_assert(kMaxBlock3 <= kPanelThreads * kPanelCtas, "rows of the widest pivot block");
+
 template <typename C, int NB>
-__global__ void __launch_bounds__(512) f3_panel(const Slab3* __restrict__ slabs, C* __restrict__ W, int* __restrict__ piv,
-                                                int* __restrict__ rowid, int j0, int Mmax, int* err) {
+__global__ void __launch_bounds__(kPanelThreads) f3_panel(const Slab3* __restrict__ slabs, C* __restrict__ W,
+                                                          int* __restrict__ piv, int* __restrict__ rowid, int j0,
+                                                          int Mmax, int* err) {
     using R = decltype(C{}.x);
+    namespace cg = cooperative_groups;
+    constexpr int NT = kPanelThreads, nw = NT / 32;
     extern __shared__ __align__(16) unsigned char smraw[];
-    C* P = reinterpret_cast<C*>(smraw);
+    C* tile = reinterpret_cast<C*>(smraw);   // NT x NB: entry q of row r at r NB + (q ^ (r % NB))
     __shared__ R red_v[32];
     __shared__ int red_i[32];
-    __shared__ C s_pj[NB], s_oj[NB], s_d;
-    __shared__ int s_pr;
-    const int slab = blockIdx.x;
+    // exchange of one pivot, two of them in turn (a CTA may be one pivot ahead)
+    __shared__ R s_val[2][kPanelCtas];
+    __shared__ int s_row[2][kPanelCtas];
+    __shared__ __align__(16) C s_new[2][kPanelCtas][NB];   // candidate rows, the pivot entry replaced by its reciprocal
+    __shared__ __align__(16) C s_old[2][NB];               // the old row j, which moves to the pivot's place
+    __shared__ __align__(16) C s_push[2][NB];
+    cg::cluster_group cl = cg::this_cluster();
+    const int ncl = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int slab = blockIdx.x / ncl;
     const Slab3 sd = slabs[slab];
     const int M = sd.M;
     if (j0 >= M) return;
     const int nbp = min(NB, M - j0);
-    C* w = W + sd.w_off;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int e = tid; e < M * nbp; e += nt) {
-        const int r = e / nbp, q = e % nbp;
-        P[q * M + r] = w[(long long)r * M + j0 + q];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int per = (M + ncl - 1) / ncl, base = rank * per, nr = max(0, min(per, M - base));
+    const int r = tid < nr ? base + tid : M;   // this thread's row
+    const int sw = tid % NB;
+    C* w = W + sd.w_off + (long long)base * M + j0;
+    for (int e = tid; e < nr * NB; e += NT) {
+        const int rr = e / NB, q = e % NB;
+        tile[rr * NB + (q ^ (rr % NB))] = q < nbp ? w[(long long)rr * M + q] : czero<C>();
     }
     __syncthreads();
-    const int nw = nt / 32;
+    C x[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) x[q] = r < M ? tile[tid * NB + (q ^ sw)] : czero<C>();
+    cl.sync();   // every CTA of the cluster runs before the first row is sent
+#pragma unroll 1
     for (int jj = 0; jj < nbp; ++jj) {
-        const int j = j0 + jj;
-        // pivot: the largest |P[jj][r]| over rows r >= j (ties to the lower row);
-        // each warp reduces its rows, then every thread reduces the warps'
-        // results itself (no second barrier)
-        R best = -1;
-        int bi = M;
-        for (int r = j + tid; r < M; r += nt) {
-            const R v = cabs2(P[jj * M + r]);
-            if (v > best) { best = v; bi = r; }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const R ov = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-        }
-        if ((tid & 31) == 0) { red_v[tid >> 5] = best; red_i[tid >> 5] = bi; }
+        const int j = j0 + jj, par = jj & 1;
+        R best = r >= j && r < M ? cabs2(x[0]) : R(0);
+        if (!(best > 0)) best = 0;   // (also NaN)
+        int bi = best > 0 ? r : M;
+        warp_pivot(best, bi);
+        if (lane == 0) { red_v[wid] = best; red_i[wid] = bi; }
         __syncthreads();
-        // warp 0: the pivot over the warps' results, the pivot row (old row pr)
-        // scaled by d = 1 / pivot and the old row j (which moves to position pr)
-        if (tid < 32) {
-            best = tid < nw ? red_v[tid] : R(-1);
-            bi = tid < nw ? red_i[tid] : M;
-            for (int o = 16; o > 0; o >>= 1) {
-                const R ov = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+        best = lane < nw ? red_v[lane] : R(0);
+        bi = lane < nw ? red_i[lane] : M;
+        warp_pivot(best, bi);
+        if (tid < ncl) {
+            *cl.map_shared_rank(&s_val[par][rank], tid) = best;
+            *cl.map_shared_rank(&s_row[par][rank], tid) = bi;
+        }
+        // the owner's warp sends the row to every CTA, NB lanes at a time
+        auto send = [&](bool mine, C head, C* buf, C* dst) {
+            if (mine) {
+                buf[0] = head;
+#pragma unroll
+                for (int q = 1; q < NB; ++q) buf[q] = x[q];
             }
-            const bool sing = !(best > 0) || !isfinite(best) || bi >= M;
-            const int pr = sing ? j : bi;
-            const C d = crecip(P[jj * M + pr]);
-            if (tid < nbp) {
-                s_pj[tid] = (tid == jj) ? d : P[tid * M + pr] * d;
-                s_oj[tid] = P[tid * M + j];
-            }
-            if (tid == 0) {
-                if (sing) atomicOr(err, LSS_DERR_SINGULAR);
-                s_pr = pr;
-                s_d = d;
-                piv[slab * NB + jj] = pr;
-                if (pr != j) {
-                    int* rid = rowid + (long long)slab * Mmax;
-                    const int t = rid[j];
-                    rid[j] = rid[pr];
-                    rid[pr] = t;
-                }
+            __syncwarp();
+            for (int e = lane; e < ncl * NB; e += 32) *cl.map_shared_rank(dst + e % NB, e / NB) = buf[e % NB];
+            __syncwarp();
+        };
+        if (bi < M && (bi - base) >> 5 == wid) send(r == bi, crecip(x[0]), s_push[0], s_new[par][rank]);
+        if (j >= base && j < base + nr && (j - base) >> 5 == wid) send(r == j, x[0], s_push[1], s_old[par]);
+        cl.sync();
+        int from = 0;
+        best = s_val[par][0];
+        bi = s_row[par][0];
+        for (int q = 1; q < ncl; ++q) {
+            const R v = s_val[par][q];
+            const int i = s_row[par][q];
+            if (v > best || (v == best && i < bi)) { best = v; bi = i; from = q; }
+        }
+        const bool sing = !(best > 0) || !isfinite(best) || bi >= M;
+        const int pr = sing ? j : bi;
+        const C* pn = sing ? s_old[par] : s_new[par][from];
+        const C d = sing ? crecip(pn[0]) : pn[0];
+        if (rank == 0 && tid == 0) {
+            if (sing) atomicOr(err, LSS_DERR_SINGULAR);
+            piv[slab * NB + jj] = pr;
+            if (pr != j) {
+                int* rid = rowid + (long long)slab * Mmax;
+                const int t = rid[j];
+                rid[j] = rid[pr];
+                rid[pr] = t;
             }
         }
-        __syncthreads();
-        // new row j = the scaled pivot row; every other row i (row pr taking
-        // the old row j's values) eliminated: x_q -= l pj_q, x_jj = -l d
-        const int pr = s_pr;
-        const C d = s_d;
-        C pj[NB];
+        // new row j = d times the pivot row; every other row (row pr taking the
+        // old row j's values) eliminated: x_q -= (x_jj d) p_q, x_jj = -x_jj d
+        if (r == j) {   // 0 + d p_q
 #pragma unroll
-        for (int q = 0; q < NB; ++q) pj[q] = q < nbp ? s_pj[q] : czero<C>();
-        for (int i = tid; i < M; i += nt) {
-            if (i == j) {
+            for (int q = 1; q < NB; ++q) x[q] = czero<C>();
+            x[0] = mk(R(-1), R(0));
+        } else if (r == pr) {
 #pragma unroll
-                for (int q = 0; q < NB; ++q)
-                    if (q < nbp) P[q * M + i] = pj[q];
-                continue;
-            }
-            const bool sw = i == pr;
-            const C l = sw ? s_oj[jj] : P[jj * M + i];
-#pragma unroll
-            for (int q = 0; q < NB; ++q) {
-                if (q >= nbp) break;
-                const C x = sw ? s_oj[q] : P[q * M + i];
-                P[q * M + i] = (q == jj) ? czero<C>() - l * d : x - l * pj[q];
-            }
+            for (int q = 0; q < NB; ++q) x[q] = s_old[par][q];
         }
-        __syncthreads();
+        const C l = czero<C>() - x[0] * d;
+#pragma unroll
+        for (int q = 1; q < NB; ++q) x[q - 1] = cfma(l, pn[q], x[q]);
+        x[NB - 1] = l;
     }
-    for (int e = tid; e < M * nbp; e += nt) {
-        const int r = e / nbp, q = e % nbp;
-        w[(long long)r * M + j0 + q] = P[q * M + r];
+    __syncthreads();
+    if (r < M)
+#pragma unroll
+        for (int q = 0; q < NB; ++q) tile[tid * NB + (((q + nbp) % NB) ^ sw)] = x[q];
+    __syncthreads();
+    for (int e = tid; e < nr * NB; e += NT) {
+        const int rr = e / NB, q = e % NB;
+        if (q < nbp) w[(long long)rr * M + q] = tile[rr * NB + (q ^ (rr % NB))];
     }
+}
+
+// Clusters of the least power of two whose threads hold every row.
+template <typename C, int NB>
+cudaError_t launch_f3_panel(int nl, const Slab3* slabs, C* W, int* piv, int* rowid, int j0, int Mmax, int* err,
+                            cudaStream_t s) {
+    int ncl = 1;
+    while (ncl * kPanelThreads < Mmax) ncl *= 2;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3(nl * ncl);
+    cfg.blockDim = dim3(kPanelThreads);
+    cfg.dynamicSmemBytes = kPanelThreads * NB * sizeof(C);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ncl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, f3_panel<C, NB>, slabs, W, piv, rowid, j0, Mmax, err);
 }
 
 // Outside the panel columns: apply the panel's row swaps; for the columns in
 // [c_lo, c_hi) also move the pivot rows' entries into T (T[jj][c], zero for c
 // in J) and zero them in W (the columns the following update covers).  The
 // swaps touch at most 2 nbp rows; their composition (row x receives the old
-// row src[x]) is worked out once per CTA, then every column is a gather: all
-// loads first, then the stores.
+// row src[x]) is worked out once per CTA, a thread per row, then every column
+// is a gather: all loads first, then the stores.
 template <typename C, int NB>
 __global__ void f3_swap_extract(const Slab3* __restrict__ slabs, C* __restrict__ W, const int* __restrict__ piv,
                                 C* __restrict__ T, int j0, int Tld, int c_lo, int c_hi) {
-    __shared__ int rows[2 * NB], src[2 * NB], nrows_s;
+    __shared__ int rows[2 * NB], src[2 * NB];   // rows[q] = -1: nothing to move
     const int slab = blockIdx.y;
     const Slab3 sd = slabs[slab];
     const int M = sd.M;
     if (j0 >= M) return;
     const int nbp = min(NB, M - j0);
-    if (threadIdx.x == 0) {
-        int na = 0;
-        for (int jj = 0; jj < nbp; ++jj) rows[na++] = j0 + jj;
-        for (int jj = 0; jj < nbp; ++jj) {
-            const int r = piv[slab * NB + jj];
-            bool seen = false;
-            for (int q = 0; q < na; ++q) seen |= rows[q] == r;
-            if (!seen) rows[na++] = r;
+    if (threadIdx.x < 2 * NB) {
+        // thread q: pivot row j0 + q, or the q-th swap's partner below the
+        // panel rows (its first mention); its source is found by undoing the
+        // swaps from the last to the first
+        const int q = threadIdx.x, *pv = piv + slab * NB;
+        int x = -1;
+        if (q < NB) {
+            if (q < nbp) x = j0 + q;
+        } else if (q - NB < nbp) {
+            x = pv[q - NB];
+            if (x < j0 + nbp) x = -1;
+            for (int u = 0; u < q - NB; ++u)
+                if (pv[u] == x) x = -1;
         }
-        for (int q = 0; q < na; ++q) src[q] = rows[q];
-        for (int jj = 0; jj < nbp; ++jj) {
-            const int r = piv[slab * NB + jj];
-            int pr = 0;
-            while (rows[pr] != r) ++pr;
-            const int tmp = src[jj];
-            src[jj] = src[pr];
-            src[pr] = tmp;
+        rows[q] = x;
+        for (int u = nbp - 1; u >= 0; --u) {
+            const int r = pv[u];
+            x = x == j0 + u ? r : x == r ? j0 + u : x;
         }
-        nrows_s = na;
+        src[q] = x;
     }
     __syncthreads();
-    const int na = nrows_s;
     C* w = W + sd.w_off;
     C* t = T + (long long)slab * NB * Tld;
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < M; c += gridDim.x * blockDim.x) {
@@ -632,11 +694,11 @@ __global__ void f3_swap_extract(const Slab3* __restrict__ slabs, C* __restrict__
         C v[2 * NB];
 #pragma unroll
         for (int q = 0; q < 2 * NB; ++q)
-            if (q < na) v[q] = w[(long long)src[q] * M + c];
+            if (rows[q] >= 0) v[q] = w[(long long)src[q] * M + c];
 #pragma unroll
         for (int q = 0; q < 2 * NB; ++q) {
-            if (q >= na) break;
-            if (q < nbp && local) {
+            if (rows[q] < 0) continue;
+            if (q < NB && local) {
                 t[(long long)q * Tld + c] = v[q];
                 w[(long long)rows[q] * M + c] = czero<C>();
             } else {
@@ -1096,7 +1158,7 @@ int configure3(lss_ctx* c) {
     if (!e) e = cudaFuncSetAttribute(mv3_cols<COL_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
     if (!e) e = cudaFuncSetAttribute(mv3_cols<COL_KHAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smax);
     const int psm = 210 * 1024;
-    const int panel = kMaxBlock3 * kNB64 * (int)sizeof(double2);   // = kMaxBlock3 * kNB32 * sizeof(float2)
+    const int panel = kPanelThreads * kNB64 * (int)sizeof(double2);   // = kPanelThreads * kNB32 * sizeof(float2)
     if (!e) e = cudaFuncSetAttribute(f3_panel<double2, kNB64>, cudaFuncAttributeMaxDynamicSharedMemorySize, panel);
     if (!e) e = cudaFuncSetAttribute(f3_panel<float2, kNB32>, cudaFuncAttributeMaxDynamicSharedMemorySize, panel);
     if (!e) e = cudaFuncSetAttribute(sweep3_kernel<double2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, psm);
@@ -1373,7 +1435,6 @@ int factor_set_t(lss_ctx* c, const FactorSet3& fs, cudaStream_t s) {
     const int ew_blocks = (int)std::min<long long>(8LL * c->num_sms / std::max(1, nl) + 1, (MM + 255) / 256);
     const int tiles = (Mmax + 63) / 64;
     const int npanel = (Mmax + NB - 1) / NB;
-    const size_t psm = (size_t)Mmax * NB * sizeof(C);
     bool use_tc = false;
     if constexpr (std::is_same<C, float2>::value) use_tc = fs.tc && lss3_use_tc();
     ProfScope ps(c, s, LSS_PROF_FACTOR, 0);
@@ -1390,7 +1451,7 @@ int factor_set_t(lss_ctx* c, const FactorSet3& fs, cudaStream_t s) {
         if (!use_tc) {
             for (int p = 0; p < npanel; ++p) {
                 const int j0 = p * NB;
-                f3_panel<C, NB><<<nl, 512, psm, s>>>(slabs, W, fs.piv, fs.rowid, j0, Mmax, c->d_err);
+                launch_f3_panel<C, NB>(nl, slabs, W, fs.piv, fs.rowid, j0, Mmax, c->d_err, s);
                 f3_swap_extract<C, NB><<<dim3((Mmax + 255) / 256, nl), 256, 0, s>>>(slabs, W, fs.piv, T, j0, Mmax,
                                                                                    0, Mmax);
                 f3_update_cc<C, NB><<<dim3(tiles * tiles, nl), 256, 0, s>>>(slabs, W, T, j0, Mmax, 0, Mmax);
@@ -1408,7 +1469,7 @@ int factor_set_t(lss_ctx* c, const FactorSet3& fs, cudaStream_t s) {
                 for (int q = 0; q < kNO / NB; ++q) {
                     const int j0 = J0 + q * NB;
                     if (j0 >= Mmax) break;
-                    f3_panel<C, NB><<<nl, 512, psm, s>>>(slabs, W, fs.piv, fs.rowid, j0, Mmax, c->d_err);
+                    launch_f3_panel<C, NB>(nl, slabs, W, fs.piv, fs.rowid, j0, Mmax, c->d_err, s);
                     f3_swap_extract<C, NB><<<dim3((Mmax + 255) / 256, nl), 256, 0, s>>>(slabs, W, fs.piv, T, j0,
                                                                                        Mmax, J0, J0 + kNO);
                     f3_update_cc<C, NB><<<dim3(tiles * otiles, nl), 256, 0, s>>>(slabs, W, T, j0, Mmax, J0,

@@ -89,7 +89,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // chain of loads, products and a read-modify-write of W, so what bounds it is
 // the warps that share an SM's latencies: 256 threads, of which one half stages
 // A while the other stages B, and the halves take alternate column chunks of
-// the epilogue.  (M = 984 .. 1476, 17 slabs: 120 us per launch with 128 threads
+// the epilogue.  (M = 984 .. 1476, 17 slabs: 87 us per launch; 120 with 128 threads
 // and the tile table of the widest slab, half of it empty, dealt round-robin.)
 constexpr int kTcThreads = 256;
 __global__ void __launch_bounds__(kTcThreads, 2) f3_update_tc(const Slab3* __restrict__ slabs, int n_slabs,
