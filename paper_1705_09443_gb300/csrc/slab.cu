@@ -247,9 +247,11 @@ constexpr int kWideThreads = 256;
 // Gauss-Jordan with partial pivoting (largest modulus in the column, lowest
 // row on ties) on [A | I | C | B] for the odd rows of level l, giving D^{-1},
 // D^{-1}C and D^{-1}B, or on [A | I] for the top row.  The augmented matrix
-// sits row-major in shared memory (row stride rs); warp 0 picks the pivot,
-// the threads swap and scale row jj column-wise, then thread (column q, row
-// parity) eliminates every other row i = parity, parity+2, ...
+// sits row-major in shared memory (row stride rs); warp 0 picks the pivot and
+// forms its reciprocal, the threads swap and scale row jj column-wise, then
+// thread (column q, row parity) eliminates every other row i = parity,
+// parity+2, ...  Three barriers a pivot; the reciprocal is one lane's, since
+// its divisions in every thread cost as much FP64 time as the elimination.
 template <typename T>
 __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __restrict__ slabs,
                                                              cx<T>* __restrict__ fac, cx<T>* __restrict__ work,
@@ -258,6 +260,7 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
     using C = cx<T>;
     extern __shared__ __align__(16) unsigned char smw[];
     __shared__ int s_piv;
+    __shared__ C s_pinv;
     const int tid = threadIdx.x, lane = tid & 31;
     const int task = blockIdx.x;
     const int si = slab0 + task / per_slab, o = task % per_slab;
@@ -295,27 +298,27 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
                 const int ob = __shfl_xor_sync(0xffffffffu, best, off);
                 if (ov > val || (ov == val && ob < best)) { val = ov; best = ob; }
             }
-            if (lane == 0) s_piv = best;
+            if (lane == best) {
+                C pv = M[best * rs + jj];
+                const T a2 = cabs2(pv);
+                if (!(a2 > T(0)) || !isfinite(a2)) {
+                    atomicOr(err, LSS_DERR_SINGULAR);
+                    pv = czero<C>();
+                    pv.x = T(1);
+                }
+                s_piv = best;
+                s_pinv = crecip(pv);
+            }
         }
         __syncthreads();
         const int r = s_piv;
-        if (r != jj)
-            for (int q = jj + tid; q < ncol; q += kWideThreads) {
-                const C t = M[jj * rs + q];
-                M[jj * rs + q] = M[r * rs + q];
-                M[r * rs + q] = t;
-            }
-        __syncthreads();
-        C pv = M[jj * rs + jj];
-        const T a2 = cabs2(pv);
-        if (!(a2 > T(0)) || !isfinite(a2)) {
-            if (tid == 0) atomicOr(err, LSS_DERR_SINGULAR);
-            pv = czero<C>();
-            pv.x = T(1);
+        const C pinv = s_pinv;
+        // rows jj and r exchanged, row jj scaled (column jj keeps the multipliers)
+        for (int q = jj + tid; q < ncol; q += kWideThreads) {
+            const C x = M[r * rs + q];
+            if (r != jj) M[r * rs + q] = M[jj * rs + q];
+            if (q > jj) M[jj * rs + q] = x * pinv;
         }
-        const C pinv = crecip(pv);
-        __syncthreads();   // every thread has read the pivot before row jj is scaled
-        for (int q = jj + 1 + tid; q < ncol; q += kWideThreads) M[jj * rs + q] = M[jj * rs + q] * pinv;
         __syncthreads();
         // column jj is not written below and not read after this pivot
         for (int q = jj + 1 + tq; q < ncol; q += 128) {
