@@ -249,8 +249,10 @@ constexpr int kWideThreads = 256;
 // D^{-1}C and D^{-1}B, or on [A | I] for the top row.  The augmented matrix
 // sits row-major in shared memory (row stride rs); warp 0 picks the pivot and
 // forms its reciprocal, the threads swap and scale row jj column-wise, then
-// thread (column q, row parity) eliminates every other row i = parity,
-// parity+2, ...  Three barriers a pivot; the reciprocal is one lane's, since
+// thread (column q, row group) eliminates rows i = group, group + npar, ...
+// Where the level has fewer rows than the SMs, three CTAs share a row: each
+// eliminates A beside one of I, C and B (the same operations on 1.5 w instead
+// of 3.5 w columns per pivot on average).  Three barriers a pivot; the reciprocal is one lane's, since
 // its divisions in every thread cost as much FP64 time as the elimination.
 template <typename T>
 __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __restrict__ slabs,
@@ -272,7 +274,9 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
     C* W = work + sd.work_off + (l & 1) * work_len;
     C* F = fac + sd.fac_off;
     const int j = top ? 0 : 2 * o + 1;
-    const int ncol = top ? 2 * w : 4 * w;
+    // parts > 1: this CTA carries only block `part` of I, C, B beside A (wd columns)
+    const int parts = gridDim.y, part = blockIdx.y;
+    const int ncol = top || parts > 1 ? 2 * w : 4 * w;
     const C* Ab = W + (long long)j * bs;
     const C* Cb = W + ((long long)K0 + 2LL * j) * bs;
     const C* Bb = Cb + bs;
@@ -280,14 +284,16 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
     for (int e = tid; e < w * ncol; e += kWideThreads) {
         const int i = e / ncol, q = e % ncol;
         C v = czero<C>();
+        const int blk = q / w - 1 + part, qb = q % w;
         if (q < w) v = Ab[(long long)q * ldw + i];
-        else if (q < 2 * w) { if (q - w == i) v.x = T(1); }
-        else if (q < 3 * w) v = Cb[(long long)(q - 2 * w) * ldw + i];
-        else if (hasB) v = Bb[(long long)(q - 3 * w) * ldw + i];
+        else if (blk == 0) { if (qb == i) v.x = T(1); }
+        else if (blk == 1) v = Cb[(long long)qb * ldw + i];
+        else if (hasB) v = Bb[(long long)qb * ldw + i];
         M[i * rs + q] = v;
     }
     __syncthreads();
-    const int tq = tid % 128, par = tid / 128;
+    const int cw = ncol <= 64 ? 64 : 128, npar = kWideThreads / cw;
+    const int tq = tid % cw, par = tid / cw;
     for (int jj = 0; jj < w; ++jj) {
         if (tid < 32) {
             T val = (lane >= jj && lane < w) ? cabs2(M[lane * rs + jj]) : T(-1);
@@ -321,9 +327,9 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
         }
         __syncthreads();
         // column jj is not written below and not read after this pivot
-        for (int q = jj + 1 + tq; q < ncol; q += 128) {
+        for (int q = jj + 1 + tq; q < ncol; q += cw) {
             const C mj = M[jj * rs + q];
-            for (int i = par; i < w; i += 2)
+            for (int i = par; i < w; i += npar)
                 if (i != jj) M[i * rs + q] = cfnma(M[i * rs + jj], mj, M[i * rs + q]);
         }
         __syncthreads();
@@ -334,15 +340,12 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
     for (int e = tid; e < bs; e += kWideThreads) {
         const int q = e / ldw, p = e % ldw;
         const bool in = p < w && q < w;
-        Dout[e] = in ? M[p * rs + w + q] : czero<C>();
-        if (!top) {
-            const C dc = in ? M[p * rs + 2 * w + q] : czero<C>();
-            const C db = in ? M[p * rs + 3 * w + q] : czero<C>();
-            DCw[e] = dc;
-            DCw[bs + e] = db;
-            if (DCf) {
-                DCf[e] = dc;
-                DCf[bs + e] = db;
+        for (int blk = part; blk < (top ? 1 : parts > 1 ? part + 1 : 3); ++blk) {
+            const C v = in ? M[p * rs + (blk - part + 1) * w + q] : czero<C>();
+            if (blk == 0) Dout[e] = v;
+            else {
+                DCw[(blk - 1) * bs + e] = v;
+                if (DCf) DCf[(blk - 1) * bs + e] = v;
             }
         }
     }
@@ -355,6 +358,8 @@ __global__ void __launch_bounds__(kWideThreads) cr_gjw_kernel(const SlabDev* __r
 // for all columns q) in shared memory; thread (column q, row group g) computes
 // rows g, g+8, g+16, g+24 of column q of A', C', B', summing over a in
 // ascending order (at level 0, where C and B are tridiagonal, over the band).
+// Two or four CTAs share a row, each with its part of those rows, where the
+// level has too few rows for the SMs.
 template <typename T>
 __global__ void __launch_bounds__(kWideThreads) cr_evenw_kernel(const SlabDev* __restrict__ slabs,
                                                                cx<T>* __restrict__ fac, cx<T>* __restrict__ work,
@@ -399,6 +404,7 @@ __global__ void __launch_bounds__(kWideThreads) cr_evenw_kernel(const SlabDev* _
     }
     __syncthreads();
     const int q = tid & 31, g = tid >> 5;
+    const int parts = gridDim.y, part = blockIdx.y;   // this CTA's u: part, part + parts, ..
     // out (rows g + 8 u) = init - L R_f for the staged left factor L
     auto product = [&](const C* L, int f, C (&out)[4]) {
         const C* R = Rt + f * 32 * LS;
@@ -406,6 +412,7 @@ __global__ void __launch_bounds__(kWideThreads) cr_evenw_kernel(const SlabDev* _
         for (int u = 0; u < 4; ++u) {
             const int pp = g + 8 * u;
             if (pp >= w) break;
+            if (u % parts != part) continue;
             C acc = czero<C>();
             if (l == 0) {
 #pragma unroll
@@ -438,6 +445,7 @@ __global__ void __launch_bounds__(kWideThreads) cr_evenw_kernel(const SlabDev* _
         for (int u = 0; u < 4; ++u) {
             const int pp = g + 8 * u;
             if (pp >= ldw) break;
+            if (u % parts != part) continue;
             const bool in = q < w && pp < w;
             const long long o = (long long)q * ldw + pp;
             An[o] = in ? oa[u] : czero<C>();
@@ -2116,9 +2124,11 @@ int factor_impl(lss_ctx* c, cudaStream_t s) {
                     cr_gj0_kernel<T><<<(nodd * u.n + kGj0Warps - 1) / kGj0Warps, 32 * kGj0Warps, 0, su>>>(
                         c->d_slabs, (const C*)c->coef, fac, work, K0, nodd, u.s0, u.n, c->d_err);
                 else
-                    cr_gjw_kernel<T><<<nodd * u.n, kWideThreads, shgw_of(u.w), su>>>(
+                    cr_gjw_kernel<T><<<dim3(nodd * u.n, 3 * nodd * u.n <= c->num_sms ? 3 : 1), kWideThreads,
+                                       shgw_of(u.w), su>>>(
                         c->d_slabs, fac, work, c->work_len, K0, l, nodd, u.s0, 0, 4 * u.w + 1, c->d_err);
-                cr_evenw_kernel<T><<<nev * u.n, kWideThreads, shew, su>>>(c->d_slabs, fac, work, c->work_len, K0,
+                const int ep = u.w <= 8 ? 1 : 4 * nev * u.n <= c->num_sms && u.w > 16 ? 4 : 2 * nev * u.n <= c->num_sms ? 2 : 1;
+                cr_evenw_kernel<T><<<dim3(nev * u.n, ep), kWideThreads, shew, su>>>(c->d_slabs, fac, work, c->work_len, K0,
                                                                          l, nev, u.s0, nlev);
             }
             cr_gjw_kernel<T><<<u.n, kWideThreads, shgw_of(u.w), su>>>(c->d_slabs, fac, work, c->work_len, K0, nlev, 1,
