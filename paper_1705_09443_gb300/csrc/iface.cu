@@ -318,22 +318,25 @@ __device__ void bwd0_body(const IfArgs<cx<T>>& A, const IfProb& pr) {
 
 // Back substitution of level l >= 1, register-tiled: the CTA stages
 // (D^{-1}C)_k, (D^{-1}B)_k and the column tiles of x_{k-s}, x_{k+s} (transposed
-// to [layer][column], rows padded to kBtN + 1 entries: conflict-free for both
+// to [layer][column], rows padded to BN + 1 entries: conflict-free for both
 // the transposing store and the column reads) in shared memory; thread
 // (row group rg, column group cg) owns layers rg*TP .. rg*TP+TP-1 of columns
 // cg + 16 t, t < TJ, and subtracts the products from y in the same order as
 // the untiled loop (block C then B, layer a ascending).
-constexpr int kBtN = 64;                 // columns per CTA
+// BN columns per CTA: 64, or 16 where a launch of 64-column tiles leaves SMs
+// idle (high levels, the few 32-wide problems): a 32-wide tile of 64 takes one
+// SM 160 us in FP64, and its launch has no more than a few rows of tiles.
+constexpr int kBtN = 64, kBtNs = 16;
 constexpr int kBtThreads = 128;          // 8 row groups x 16 column groups
 constexpr int kBtNP = kBtN + 1;
 
-template <typename T, int G>
+template <typename T, int G, int BN>
 __device__ void bwd_tiled_body(const IfArgs<cx<T>>& A, const IfProb& pr, int l) {
     using C = cx<T>;
-    constexpr int RG = 8, CGN = 16, TP = G / RG, TJ = kBtN / CGN;
+    constexpr int RG = 8, CGN = 16, TP = G / RG, TJ = BN / CGN, BNP = BN + 1;
     extern __shared__ __align__(16) unsigned char smi[];
     C* Ms = reinterpret_cast<C*>(smi);   // [2][G * G], column-major blocks
-    C* Xs = Ms + 2 * G * G;              // [2][G][kBtNP]
+    C* Xs = Ms + 2 * G * G;              // [2][G][BNP]
     const int K = A.K;
     const SlabDev sd = A.slabs[pr.slab];
     const int bs = G * G;
@@ -343,9 +346,9 @@ __device__ void bwd_tiled_body(const IfArgs<cx<T>>& A, const IfProb& pr, int l) 
     const int r = blockIdx.y;
     if (r >= lv.K / 2) return;
     const int k = (2 * r + 1) * s;
-    const int j0 = blockIdx.x * kBtN;
+    const int j0 = blockIdx.x * BN;
     if (j0 >= K) return;
-    const int nj = min(kBtN, K - j0);
+    const int nj = min(BN, K - j0);
     const int nb = k + s < K ? 2 : 1;
     C* X = A.X + pr.xoff;
     const int tid = threadIdx.x;
@@ -353,8 +356,8 @@ __device__ void bwd_tiled_body(const IfArgs<cx<T>>& A, const IfProb& pr, int l) 
     for (int e = tid; e < nb * bs; e += kBtThreads) Ms[e] = Mg[e];
     for (int b = 0; b < nb; ++b) {
         const C* src = X + ((long long)(b == 0 ? k - s : k + s) * K + j0) * G;
-        C* dst = Xs + b * G * kBtNP;
-        for (int e = tid; e < nj * G; e += kBtThreads) dst[(e % G) * kBtNP + e / G] = src[e];
+        C* dst = Xs + b * G * BNP;
+        for (int e = tid; e < nj * G; e += kBtThreads) dst[(e % G) * BNP + e / G] = src[e];
     }
     const int rg = tid / CGN, cg = tid % CGN;
     const int ylo = win_lo(k, l), yhi = win_hi(k, l, K);
@@ -370,14 +373,14 @@ __device__ void bwd_tiled_body(const IfArgs<cx<T>>& A, const IfProb& pr, int l) 
     __syncthreads();
     for (int b = 0; b < nb; ++b) {
         const C* M = Ms + b * bs + rg * TP;
-        const C* Xb = Xs + b * G * kBtNP + cg;
+        const C* Xb = Xs + b * G * BNP + cg;
 #pragma unroll 4
         for (int a = 0; a < G; ++a) {
             C m[TP], x[TJ];
 #pragma unroll
             for (int q = 0; q < TP; ++q) m[q] = M[a * G + q];
 #pragma unroll
-            for (int t = 0; t < TJ; ++t) x[t] = Xb[a * kBtNP + CGN * t];
+            for (int t = 0; t < TJ; ++t) x[t] = Xb[a * BNP + CGN * t];
 #pragma unroll
             for (int q = 0; q < TP; ++q)
 #pragma unroll
@@ -394,11 +397,11 @@ __device__ void bwd_tiled_body(const IfArgs<cx<T>>& A, const IfProb& pr, int l) 
     }
 }
 
-template <typename T>
+template <typename T, int BN>
 __global__ void __launch_bounds__(kBtThreads) if_bwdt_kernel(IfArgs<cx<T>> A, int l, int zoff) {
     const IfProb pr = A.probs[zoff + blockIdx.z];
-    if (pr.G == 16) bwd_tiled_body<T, 16>(A, pr, l);
-    else bwd_tiled_body<T, 32>(A, pr, l);
+    if (pr.G == 16) bwd_tiled_body<T, 16, BN>(A, pr, l);
+    else bwd_tiled_body<T, 32, BN>(A, pr, l);
 }
 
 template <typename T>
@@ -576,7 +579,7 @@ int iface_impl(lss_ctx* c, cudaStream_t s) {
     }
     const size_t sht = sizeof(C) * ((size_t)2 * gmax * gmax + (size_t)2 * gmax * kBtNP);
     const size_t sh0 = sizeof(T) == 4 ? sizeof(C) * (size_t)kB0N * (gmax + 1) : 0;
-    long long& cfg_t = lss_dev_cache((const void*)if_bwdt_kernel<T>, 0);
+    long long& cfg_t = lss_dev_cache((const void*)if_bwdt_kernel<T, kBtN>, 0);
     long long& cfg_0 = lss_dev_cache((const void*)if_bwd0_kernel<T>, 0);
     if (sizeof(T) == 4 && (long long)sh0 > cfg_0) {
         cudaError_t e = cudaFuncSetAttribute(if_bwd0_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -585,8 +588,9 @@ int iface_impl(lss_ctx* c, cudaStream_t s) {
         cfg_0 = (long long)sh0;
     }
     if ((long long)sht > cfg_t) {
-        cudaError_t e = cudaFuncSetAttribute(if_bwdt_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)std::max<size_t>(sht, 48 * 1024));
+        const int most = (int)std::max<size_t>(sht, 48 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(if_bwdt_kernel<T, kBtN>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (!e) e = cudaFuncSetAttribute(if_bwdt_kernel<T, kBtNs>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e) return lss_check_cuda(c, e, "interface attribute");
         cfg_t = (long long)sht;
     }
@@ -618,12 +622,18 @@ int iface_impl(lss_ctx* c, cudaStream_t s) {
         cudaStreamWaitEvent(c->aux_stream[0], c->fork_event, 0);
     }
     cudaStream_t s32 = two ? c->aux_stream[0] : s;
-    const size_t sh16 = sizeof(C) * ((size_t)2 * 16 * 16 + (size_t)2 * 16 * kBtNP);
+    auto bwdt = [&](int G, int l, int count, int zoff, cudaStream_t st) {
+        const int rows = std::max(1, cr_level(K, l).K / 2);
+        const bool small = (long long)ktt * rows * count < c->num_sms;
+        const int bn = small ? kBtNs : kBtN;
+        const size_t shb = sizeof(C) * ((size_t)2 * G * G + (size_t)2 * G * (bn + 1));
+        const dim3 grid((K + bn - 1) / bn, rows, count);
+        if (small) if_bwdt_kernel<T, kBtNs><<<grid, kBtThreads, shb, st>>>(A, l, zoff);
+        else if_bwdt_kernel<T, kBtN><<<grid, kBtThreads, shb, st>>>(A, l, zoff);
+    };
     for (int l = L - 1; l > 0; --l) {
-        const int Kl = cr_level(K, l).K;
-        if (n16 > 0) if_bwdt_kernel<T><<<dim3(ktt, std::max(1, Kl / 2), n16), kBtThreads, sh16, s>>>(A, l, 0);
-        if (np > n16)
-            if_bwdt_kernel<T><<<dim3(ktt, std::max(1, Kl / 2), np - n16), kBtThreads, sht, s32>>>(A, l, n16);
+        if (n16 > 0) bwdt(16, l, n16, 0, s);
+        if (np > n16) bwdt(32, l, np - n16, n16, s32);
     }
     if (two) {
         cudaEventRecord(c->aux_event[0], s32);
