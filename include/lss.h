@@ -391,6 +391,10 @@ int lss_batch_instance(lss_ctx *c, int q, lss_ctx **inst);
  *             satisfies (a grid barrier one arrival short, an mbarrier nobody
  *             arrives at); each gives up after the wait limit (about 2 s) and
  *             the call returns LSS_ERR_TIMEOUT; the context stays usable
+ *   what = 3  (3D, mixed precision) run the factorization's tensor-core update
+ *             on zeroed arrays with its product waits reported as expired by
+ *             half of each CTA's warps: every CTA gives up as a whole and the
+ *             call returns LSS_ERR_TIMEOUT; the factors are not touched
  * Returns LSS_ERR_ARG for other values or on a batch context.
  */
 int lss_test_inject(lss_ctx *c, int what, int a, long long b, void *stream);

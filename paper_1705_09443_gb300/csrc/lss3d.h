@@ -113,7 +113,7 @@ int lss3r_factor(lss_ctx* c, cudaStream_t s);
 int lss3r_sweep(lss_ctx* c, const double2* r, double2* y, int R, int only, const double2* fin, cudaStream_t s);
 void lss3r_free(lss_ctx* c);
 // tc_update.cu: rank-16 Gauss-Jordan update of the FP32 pivot blocks on the tensor cores (3xTF32)
-int lss3_update_tc(lss_ctx* c, float2* W, const float2* T64, int J0, int NO, cudaStream_t s);
+int lss3_update_tc(lss_ctx* c, float2* W, const float2* T64, int J0, int NO, cudaStream_t s, bool expire = false);
 bool lss3_use_tc();
 
 // greens.cu: cyclic Jacobi eigen-decomposition of a real symmetric matrix

@@ -620,6 +620,22 @@ int lss_test_inject(lss_ctx* c, int what, int a, long long b, void* stream) {
         if (rc) return rc;
         return lss_check_device_err(c, s);
     }
+    if (what == 3) {   // the tensor-core update with waits that expire for half of the warps, on zeroed arrays
+        if (c->dim != 3 || c->prec == LSS_FP64) return lss_fail(c, LSS_ERR_ARG, "test_inject: needs a 3D mixed context");
+        constexpr int NO = 64;   // panel columns
+        long long len = 0;
+        for (const Slab3& sd : c->d3->slabs) len = std::max(len, sd.w_off + (long long)sd.M * sd.M);
+        const size_t wb = (size_t)len * sizeof(float2), tb = (size_t)c->n_slabs * NO * c->d3->Mmax * sizeof(float2);
+        char* buf = nullptr;
+        int rc = dalloc(c, (void**)&buf, wb + tb, "test update");
+        if (rc) return rc;
+        rc = lss_check_cuda(c, cudaMemsetAsync(buf, 0, wb + tb, s), "test update");
+        if (!rc) rc = lss3_update_tc(c, (float2*)buf, (const float2*)(buf + wb), 0, NO, s, true);
+        const int rs = lss_check_cuda(c, cudaStreamSynchronize(s), "update self-test");
+        cudaFree(buf);
+        if (rc || rs) return rc ? rc : rs;
+        return lss_check_device_err(c, s);
+    }
     return lss_fail(c, LSS_ERR_ARG, "test_inject: unknown injection");
 }
 

@@ -91,7 +91,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // A while the other stages B, and the halves take alternate column chunks of
 // the epilogue.  (M = 984 .. 1476, 17 slabs: 87 us per launch; 120 with 128 threads
 // and the tile table of the widest slab, half of it empty, dealt round-robin.)
+// The bounded wait can expire for some threads and not for others, and the
+// halves meet on barriers of their own: whether the CTA goes on is decided for
+// all its threads together.  EXPIRE: every second warp reports its first wait
+// as expired (fault injection).
 constexpr int kTcThreads = 256;
+template <bool EXPIRE>
 __global__ void __launch_bounds__(kTcThreads, 2) f3_update_tc(const Slab3* __restrict__ slabs, int n_slabs,
                                                      float2* __restrict__ W, const float2* __restrict__ T64, int J0,
                                                      int NO, int Tld, int* err) {
@@ -210,11 +215,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) f3_update_tc(const Slab3* __res
                              smem_u32(bar))
                          : "memory");
         }
-        if (!mbar_wait(bar, phase, err)) ok = false;
+        ok = mbar_wait(bar, phase, err);
+        if (EXPIRE && (warp & 1)) {
+            ok = false;
+            if ((tid & 31) == 0) atomicOr(err, LSS_DERR_TIMEOUT);
+        }
         phase ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // the next chunk's operand writes must not overtake this chunk's products
-        __syncthreads();
+        ok = __syncthreads_and(ok);
         }   // K chunks
         if (!ok) break;
 
@@ -265,14 +274,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) f3_update_tc(const Slab3* __res
 }  // namespace
 
 // Launches the tensor-core update for the outer panel [J0, J0 + NO) of every
-// slab (FP32 factors).
-int lss3_update_tc(lss_ctx* c, float2* W, const float2* T64, int J0, int NO, cudaStream_t s) {
+// slab (FP32 factors).  expire: with waits that report expiry (fault injection).
+int lss3_update_tc(lss_ctx* c, float2* W, const float2* T64, int J0, int NO, cudaStream_t s, bool expire) {
     Ctx3* d = c->d3;
+    auto kern = expire ? f3_update_tc<true> : f3_update_tc<false>;
     {
         std::lock_guard<std::mutex> lock(lss_config_mutex());
-        long long& done = lss_dev_cache((const void*)f3_update_tc, 0);
+        long long& done = lss_dev_cache((const void*)kern, 0);
         if (!done) {
-            cudaError_t e = cudaFuncSetAttribute(f3_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
             if (e) return lss_check_cuda(c, e, "tensor-core update attribute");
             done = 1;
         }
@@ -281,7 +291,7 @@ int lss3_update_tc(lss_ctx* c, float2* W, const float2* T64, int J0, int NO, cud
     for (const Slab3& sd : d->slabs)
         if (J0 < sd.M) tiles += ((sd.M + 127) / 128) * ((sd.M + 127) / 128);
     const int grid = std::max(1, std::min(tiles, 2 * c->num_sms));
-    f3_update_tc<<<grid, kTcThreads, kTcSmem, s>>>(d->d_slabs, c->n_slabs, W, T64, J0, NO, d->Mmax, c->d_err);
+    kern<<<grid, kTcThreads, kTcSmem, s>>>(d->d_slabs, c->n_slabs, W, T64, J0, NO, d->Mmax, c->d_err);
     return lss_check_cuda(c, cudaGetLastError(), "tensor-core update launch");
 }
 

@@ -163,7 +163,8 @@ class LSSolver:
     def test_inject(self, what: int, a: int = 0, b: int = 0, stream=None):
         """Fault injection for tests (lss_test_inject): 1 = zero block row b of
         slab a (the next factor meets a zero pivot), 2 = bounded device waits
-        that expire (returns LSS_ERR_TIMEOUT)."""
+        that expire (returns LSS_ERR_TIMEOUT), 3 = the 3D mixed tensor-core update
+        with waits that expire for half of the warps (LSS_ERR_TIMEOUT)."""
         self._check(self.lib.lss_test_inject(self.ctx, int(what), int(a), int(b), _stream_ptr(stream)))
 
     def solve(self, g: torch.Tensor, opts: GmresOptions | None = None, stream=None, raise_on_noconv=True):
