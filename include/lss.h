@@ -160,6 +160,12 @@ int lss_plane_wave_rhs(lss_ctx *c, const double *dirs_host, int R, void *g_dev,
  * lss_apply_A - y = (I + omega^2 K M) x (transpose = 0) or
  * y = (I + omega^2 M K) x = A^T x (transpose = 1), Eq. LS_d_c, for R vectors;
  * zero-padded FFT convolution.  x_dev and y_dev may not alias.
+ * In both precisions of a context the operator is exact to double rounding.
+ * With padded lines of 64 to 2048 entries (n from 17 to 1024, in 3D to 128) the
+ * transforms run in 64-bit fixed point, one exponent per line: the convolution's
+ * error relative to its 2-norm is 1e-16 to 2e-16, not above that of FP64
+ * transforms, and spread evenly over the field; an entry's own error is a
+ * fraction of its line's largest entry.
  */
 int lss_apply_A(lss_ctx *c, const void *x_dev, void *y_dev, int R, int transpose,
                 void *stream);

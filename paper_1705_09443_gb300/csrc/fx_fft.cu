@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(FxPlan<LG, E>::TPB, fx_min_ctas(FxPlan<LG, E>:
 }
 
 // One CTA per line of the kernel transform (storage order): its largest part
-// sets the exponent, the entries become digits below 2^61.
+// sets the exponent of the line's digits.
 template <int LG>
 __global__ void __launch_bounds__(128) fx_khat_kernel(const double2* __restrict__ khat, fx_tw* __restrict__ out,
                                                       int* __restrict__ ek, int dim) {
@@ -276,17 +276,12 @@ __global__ void __launch_bounds__(128) fx_khat_kernel(const double2* __restrict_
     }
     atomicMax(&big, e);
     __syncthreads();
-    const int x = max((int)big, 64) - 1022 - 61;   // parts are below 2^(x + 61)
+    const int x = fx_kernel_exp(big);
     if (threadIdx.x == 0) ek[line] = x;
     for (int s = threadIdx.x; s < L; s += blockDim.x) {
         const double2 k = khat[src + fx_freq<LG, kFxBase>(s)];
-        long long q[2] = {__double2ll_rn(scalbn(k.x, -x)), __double2ll_rn(scalbn(k.y, -x))};
-        fx_digits d[2];
-        for (int i = 0; i < 2; ++i) {
-            d[i] = fx_split(q[i]);
-            if (d[i].lo == (int)0x80000000) d[i].lo += 1;   // its negative has to be a digit too
-        }
-        out[(long long)line * L + s] = fx_tw{d[0].hi, d[0].lo, d[1].hi, d[1].lo};
+        out[(long long)line * L + s] =
+            fx_kernel_digits(__double2ll_rn(scalbn(k.x, -x)), __double2ll_rn(scalbn(k.y, -x)));
     }
 }
 

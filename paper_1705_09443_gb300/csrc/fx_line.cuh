@@ -3,19 +3,28 @@
 // This GPU issues 1.6 FP64 operations per clock and SM but about 24 32 x 32 ->
 // 64-bit integer multiply-adds and 110 integer adds (measured): an FFT in
 // 64-bit integers takes a fraction of the FP64 pipe's time, which bounded the
-// operator (n = 512, 64 right-hand sides: 13.4 -> 2.95 ms; 3D n = 64: 365 ->
-// 117 us).  A line is held as integers with one exponent, v * 2^E, scaled so
+// operator (n = 512, 64 right-hand sides: 13.4 -> 3.24 ms; 3D n = 64: 365 ->
+// 136 us).  A line is held as integers with one exponent, v * 2^E, scaled so
 // that its largest entry uses the bits that a pass's growth leaves free:
 //  - additions are exact,
 //  - the product with a twiddle factor (2^62 exp(-2 pi i k / L)) keeps the high
 //    64 bits, rounded, so every factor between two passes also scales by 1/4,
 //  - between two passes the line is shifted so that its largest entry has
 //    60 or 61 - lg(radix) bits (the largest entry is an OR over the line,
-//    formed on the way through shared memory), whatever the line grew by.
-// The error of the convolution relative to the 2-norm of its result is
-// 1.9e-16 (L = 512), 2.3e-16 (1024) and 2.1e-16 (2048) against 2.4e-16,
-// 2.6e-16 and 2.9e-16 of the FP64 transforms, both against 80-bit arithmetic
-// on wave fields.
+//    formed on the way through shared memory), whatever the line grew by,
+//  - every rounding is to nearest, ties to even.  An entry is an integer, so
+//    ties are common (a quarter of the entries where a factor is 1); rounded
+//    up, or the fraction of a product dropped, the mean error of an entry is
+//    not zero and adds up at index 0 of the inverse transform (n = 200, noise:
+//    first row 1.3e-15 of the field against 1.5e-16 in the others; now 1.0e-16
+//    in all).  It costs 8 to 10 % of the operator (n = 512: 2.98 -> 3.24 ms).
+// The error of the convolution relative to the 2-norm of its result is, on wave
+// fields against 80-bit arithmetic, 1.5e-16 (L = 512), 1.8e-16 (1024) and
+// 1.9e-16 (2048); that of FP64 transforms 2.3e-16, 3.1e-16 and 2.8e-16.  An
+// entry's own error is a fraction of its line's largest entry, where FP64's is
+// one of the entry: it was compared row by row and for fields whose transform
+// is concentrated (constant, alternating in sign, rows from 1 to 1e-12), and
+// is below FP64's in all of them (tests/fixed_fft_host.cu).
 // Non-finite input marks its line (exponent kFxBad) and through it every
 // line that reads it, so the result is NaN as in floating point.
 #pragma once
@@ -52,9 +61,11 @@ struct __align__(16) fx_tw { int ch, cl, sh, sl; };
 
 // (h 2^32 + m) / 2^32 rounded, where m is kept as m + 2^63 + 2^31 and h as
 // h - 2^31: the middle sum is then unsigned and its high word needs no sign.
+// Its low word is zero on a tie (factors 1, i, -1, -i), which goes to even.
 constexpr long long kFxMid = (long long)0x8000000080000000ull, kFxTop = -0x80000000ll;
 FX_HD long long fx_join(long long h, long long m) {
-    return (long long)((unsigned long long)h + ((unsigned long long)m >> 32));
+    const unsigned long long r = (unsigned long long)h + ((unsigned long long)m >> 32);
+    return (long long)(r & ~(unsigned long long)((unsigned)m == 0));
 }
 
 // w x / 2^64, rounded; the product of the two low digits (below one unit) is
@@ -95,7 +106,8 @@ FX_HD long long fx_rsqrt2(long long v) {
 }
 FX_HD fx2 fx_mul_w8(fx2 a) { return {fx_rsqrt2(a.x + a.y), fx_rsqrt2(a.y - a.x)}; }        // a exp(-i pi/4)
 FX_HD fx2 fx_mul_w8_3(fx2 a) { return {fx_rsqrt2(a.y - a.x), fx_rsqrt2(-a.x - a.y)}; }     // a exp(-3 i pi/4)
-FX_HD fx2 fx_quarter(fx2 a) { return {(a.x + 2) >> 2, (a.y + 2) >> 2}; }
+FX_HD long long fx_quarter(long long v) { return (v + 1 + ((v >> 2) & 1)) >> 2; }
+FX_HD fx2 fx_quarter(fx2 a) { return {fx_quarter(a.x), fx_quarter(a.y)}; }
 
 FX_HD void fx_dft4(fx2& a, fx2& b, fx2& c, fx2& d) {
     const fx2 s = a + c, t = a - c, u = b + d, w = fx_mul_mi(b - d);
@@ -286,11 +298,11 @@ FX_HD void fx_inv_pass(fx2* v, int t, const typename FxPlan<LG, E>::Tw* __restri
     }
 }
 
-// v 2^s, rounded
+// v 2^s, rounded (ties to even)
 FX_HD long long fx_shift(long long v, int s) {
     if (s >= 0) return (long long)((unsigned long long)v << (s & 63));
     const int b = -s > 62 ? 62 : -s;
-    return ((v >> (b - 1)) + 1) >> 1;
+    return (v + ((1ll << (b - 1)) - 1) + ((v >> b) & 1)) >> b;
 }
 // The shift of a whole line (0 <= s < 32 but for the rare line that grew)
 template <int E>
@@ -334,16 +346,33 @@ FX_HD long long fx_from_double(double d, int& e) {
     return b < 0 ? -v : v;
 }
 
-// Product with a kernel-transform entry: w = (v k) >> 64 with the next 32 bits
-// in frac, shifted right by PS.
+// Kernel-transform entries: digits below 2^61 with one exponent per line, 2^x
+// per unit (field: the exponent field of the line's largest part).
+FX_HD int fx_kernel_exp(unsigned field) { return (field > 64 ? (int)field : 64) - 1022 - 61; }
+FX_HD fx_tw fx_kernel_digits(long long re, long long im) {
+    fx_digits a = fx_split(re), b = fx_split(im);
+    if (a.lo == (int)0x80000000) a.lo += 1;   // its negative has to be a digit too
+    if (b.lo == (int)0x80000000) b.lo += 1;
+    return {a.hi, a.lo, b.hi, b.lo};
+}
+
+// Product with a kernel-transform entry: w = (v k) >> 64 with 16 more bits in
+// the upper half of frac, shifted right by PS.  The bits below those are folded
+// into the last of the 16 (rounding to odd, so that fx_lift's rounding is that
+// of the product; the lower half is not to be used).  The products of the low digits count here: an entry that the
+// kernel makes small is shifted up afterwards, by many bits where the line's
+// energy lies far from its resonance (n = 512, a field of alternating sign:
+// error 1.3e-16 against 5.4e-15 without them, 6.2e-16 in FP64).
 template <int PS>
 FX_HD void fx_kmul(fx2 v, fx_tw k, fx2& w, unsigned& fx, unsigned& fy) {
     const fx_digits r = fx_split(v.x), i = fx_split(v.y);
-    long long a = fx_mad(r.hi, k.cl, 0);
+    long long a = fx_mad(r.lo, k.cl, fx_mad(i.lo, -k.sl, 0)) >> 32;
+    a = fx_mad(r.hi, k.cl, a);
     a = fx_mad(r.lo, k.ch, a);
     a = fx_mad(i.hi, -k.sl, a);
     a = fx_mad(i.lo, -k.sh, a);
-    long long b = fx_mad(r.hi, k.sl, 0);
+    long long b = fx_mad(r.lo, k.sl, fx_mad(i.lo, k.cl, 0)) >> 32;
+    b = fx_mad(r.hi, k.sl, b);
     b = fx_mad(r.lo, k.sh, b);
     b = fx_mad(i.hi, k.cl, b);
     b = fx_mad(i.lo, k.ch, b);
@@ -351,9 +380,13 @@ FX_HD void fx_kmul(fx2 v, fx_tw k, fx2& w, unsigned& fx, unsigned& fy) {
     const long long y = fx_mad(r.hi, k.sh, fx_mad(i.hi, k.ch, b >> 32));
     fx = (unsigned)((((unsigned long long)(unsigned)x << 32) | (unsigned)a) >> PS);
     fy = (unsigned)((((unsigned long long)(unsigned)y << 32) | (unsigned)b) >> PS);
+    fx |= (unsigned)((fx & 0xffffu) != 0) << 16;
+    fy |= (unsigned)((fy & 0xffffu) != 0) << 16;
     w = {x >> PS, y >> PS};
 }
-// (w : frac) 2^s without the bits below one unit, 0 <= s < 32
+// (w : frac) 2^s rounded to units, ties to even; 0 <= s < 32, frac a multiple of 2^16
 FX_HD long long fx_lift(long long w, unsigned frac, int s) {
-    return (long long)((unsigned long long)w << s) | (long long)(((unsigned long long)frac << s) >> 32);
+    const unsigned long long f = (unsigned long long)frac << s;
+    const long long v = (long long)(((unsigned long long)w << s) + (f >> 32));
+    return v + ((unsigned)f + (unsigned)(v & 1) > 0x80000000u);
 }
