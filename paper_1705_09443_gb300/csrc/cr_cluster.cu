@@ -501,12 +501,17 @@ int launch(lss_ctx* c, CrcArgs A, int nsl, cudaStream_t s) {
     // 32-wide slabs are few and four times the work, so theirs is the longest
     // chain: 8 CTAs (FP64 n = 256, 1: 1000 us, with 4 1070 and with 2 1490;
     // clusters of 16 take longer in mixed precision, n = 256: 360 us against 200).
+    // Beside a block LU of the other slabs the SMs are not theirs alone: 4 CTAs
+    // of more than 32 rows each (P, mixed, ms, with 8 / 4 / 2 CTAs: n = 64, 64
+    // right-hand sides 1.47 / 1.47 / 1.39, n = 128, 64 3.31 / 3.08 / 3.07 and 96
+    // 1.36 / 1.30 / 1.43, n = 256, 32 2.13 / 1.95 / 1.95).
     int cl = 1;
     if (G == 16) {
         while (cl < 4 && K > 4 * cl && ((long long)total * groups * cl < c->num_sms * 3 / 4 || K / (2 * cl) >= 128))
             cl *= 2;
     } else {
-        while (cl < 8 && K > 4 * cl && (long long)total * groups * cl < c->num_sms) cl *= 2;
+        const int most = A.beside ? 4 : 8, rows = A.beside ? 64 : 4;
+        while (cl < most && K > rows * cl && (long long)total * groups * cl < c->num_sms) cl *= 2;
     }
     // two CTAs per SM for the 16-wide slabs; past 8 CTAs only where the rows fit no other way
     while (cl < 8 && smem((K + cl - 1) / cl) > (G == 16 ? kCrcSmem / 2 : kCrcSmem)) cl *= 2;

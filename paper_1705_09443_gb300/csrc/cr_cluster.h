@@ -17,6 +17,7 @@ struct CrcArgs {
     double2* y;              // forward CRC_E output, R x n^2 (or R x n_tot^2 when y_grid)
     int y_grid;
     void* X;                 // transposed CRC_E output: R x n_tot^2 grid, x2 index slowest
+    int beside;              // the pass's 16-wide slabs run beside this launch (block LU)
     // filled by lss_cr_cluster
     const SlabDev* slabs;
     int n_slabs, n_tot, n, b, slab0, L, P;

@@ -2026,7 +2026,10 @@ size_t thomas_scratch(const lss_ctx* c, int nsl, int R) {
 }
 
 // The 16-wide runs go to the block LU when the caller prepared its factors,
-// everything else to the cyclic reduction on clusters.
+// everything else to the cyclic reduction on clusters.  The clusters are issued
+// first, on the caller's stream: a cluster needs its SMs free at the same time,
+// and behind a block LU that fills the GPU it starts when that ends (mixed,
+// n = 512, 20 right-hand sides, two fronts: 2.69 ms of pass A against 1.40).
 template <typename T, int MODE>
 int sweep_pass(lss_ctx* c, CrArgs<cx<T>> A, int R, cudaStream_t s, bool thomas = false) {
     const std::vector<SweepRun> runs = sweep_runs(c);
@@ -2049,16 +2052,20 @@ int sweep_pass(lss_ctx* c, CrArgs<cx<T>> A, int R, cudaStream_t s, bool thomas =
     Q.phi = A.phi;
     Q.y = A.y;
     Q.y_grid = A.y_grid;
+    Q.beside = qtot != 0;
+    std::vector<size_t> order(runs.size());
+    for (size_t ri = 0; ri < runs.size(); ++ri) order[ri] = ri;
+    std::stable_partition(order.begin(), order.end(), [&](size_t q) { return !th_run(runs[q]); });
     if (runs.size() > 1) cudaEventRecord(c->fork_event, s);
     for (size_t ri = 0; ri < runs.size() && !rc; ++ri) {
-        const SweepRun& u = runs[ri];
+        const SweepRun& u = runs[order[ri]];
         cudaStream_t su = ri == 0 ? s : c->aux_stream[ri - 1];
         if (ri > 0) cudaStreamWaitEvent(su, c->fork_event, 0);
         if (th_run(u)) {
             if constexpr (sizeof(T) == 4) {
                 CrArgs<cx<T>> Ar = A;
                 Ar.slab0 = u.s0;
-                rc = launch_thomas<T, MODE>(c, Ar, u.n, R, su, qoff[ri]);
+                rc = launch_thomas<T, MODE>(c, Ar, u.n, R, su, qoff[order[ri]]);
             }
         } else {
             rc = lss_cr_cluster(c, MODE == CR_A ? CRC_A : CRC_E, false, Q, u.s0, u.n, u.ldw, su);
