@@ -247,8 +247,10 @@ int lss_matvec(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int
     return lss_check_cuda(c, cudaGetLastError(), "matvec launch");
 }
 
-// kc: L x L circular kernel table (device).  khatT = omega^2/L^2 * FFT2(kc), transposed.
-int lss_fft_kernel_table(lss_ctx* c, const double2* kc, cudaStream_t s) {
+// kc: L x L circular kernel table (device).  khatT = omega^2/L^2 * FFT2(kc),
+// transposed; for the fixed-point lengths its digits take khatT's place and kc
+// is overwritten.
+int lss_fft_kernel_table(lss_ctx* c, double2* kc, cudaStream_t s) {
     const int L = c->L, lg = c->lgL;
     int rc = lss_grow(c, (void**)&c->mv_buf, &c->mv_cap, (size_t)L * L * sizeof(double2));
     if (rc) return rc;
@@ -259,15 +261,14 @@ int lss_fft_kernel_table(lss_ctx* c, const double2* kc, cudaStream_t s) {
                                                      L, lg, c->omega, c->h);
     const int C = col_group(L);
     const double scale = c->omega * c->omega / ((double)L * (double)L);
+    const bool fx = lss_fx_supported(lg);
     mv_cols<false><<<dim3(L / C, 1), C * nt, 2 * (size_t)C * L * sizeof(double2), s>>>(
-        c->mv_buf, nullptr, c->khatT, c->tw, L, L, lg, C, scale);
+        c->mv_buf, nullptr, fx ? kc : c->khatT, c->tw, L, L, lg, C, scale);
     rc = lss_check_cuda(c, cudaGetLastError(), "kernel table fft");
-    if (!rc && lss_fx_supported(lg)) {
-        rc = lss_fx_tables(c, c->khatT, s);
-        if (!rc) {
-            cudaFree(c->khatT);
-            c->khatT = nullptr;
-        }
+    if (!rc && fx) {
+        c->fx_khat = c->khatT;
+        c->khatT = nullptr;
+        rc = lss_fx_tables(c, kc, s);
     }
     return rc;
 }

@@ -387,27 +387,24 @@ int lss_fx_tables(lss_ctx* c, const double2* khat, cudaStream_t s) {
                   FxPlan<11, 8>::kThree == false, "twiddle forms below");
     const bool three = lg >= 8 && lg <= 10;   // FxPlan::kThree
     const size_t tws = three ? sizeof(fx_tw3) : sizeof(fx_tw);
-    std::vector<fx_tw3> tw3(L);
-    std::vector<fx_tw> tw(L);
+    c->fx_host.resize(L * tws / sizeof(int));
+    std::vector<long double> re(L), im(L);
+    fx_host_roots(L, re.data(), im.data());
     for (int k = 0; k < L; ++k) {
-        const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)L;
-        fx_host_tw(cosl(a), sinl(a), tw3[k]);
-        fx_host_tw(cosl(a), sinl(a), tw[k]);
+        if (three) fx_host_tw(re[k], im[k], ((fx_tw3*)c->fx_host.data())[k]);
+        else fx_host_tw(re[k], im[k], ((fx_tw*)c->fx_host.data())[k]);
     }
-    const void* twp = three ? (const void*)tw3.data() : (const void*)tw.data();
-    cudaError_t e = cudaMalloc(&c->fx_tw, L * tws);
-    if (!e) e = cudaMalloc(&c->fx_khat, lines * L * sizeof(fx_tw));
-    if (!e) e = cudaMalloc((void**)&c->fx_ek, lines * sizeof(int));
+    cudaError_t e = cudaMalloc(&c->fx_tw, L * tws + lines * sizeof(int));
     if (e) {
         cudaGetLastError();
         return lss_fail(c, LSS_ERR_OOM, "device allocation failed: fixed-point operator tables");
     }
-    e = cudaMemcpyAsync(c->fx_tw, twp, L * tws, cudaMemcpyHostToDevice, s);
+    c->fx_ek = (int*)((char*)c->fx_tw + L * tws);
+    e = cudaMemcpyAsync(c->fx_tw, c->fx_host.data(), L * tws, cudaMemcpyHostToDevice, s);
     if (!e) {
         ProfScope ps(c, s, LSS_PROF_SETUP, 1);
         e = khat_digits(lg, c->dim, khat, (fx_tw*)c->fx_khat, c->fx_ek, s);
     }
-    if (!e) e = cudaStreamSynchronize(s);   // tw is read until here; the caller frees khat
     return lss_check_cuda(c, e, "fixed-point operator tables");
 }
 

@@ -4,6 +4,7 @@
 #include <complex>
 #include <vector>
 
+#include "fx_line.cuh"
 #include "lss_common.cuh"
 #include "lss_ctx.h"
 #include "lss3d.h"
@@ -254,10 +255,9 @@ void lss_jacobi_eigen(std::vector<double> A, int n, std::vector<double>& d, std:
 int lss_build_kernel(lss_ctx* c, cudaStream_t s) {
     const int L = c->L;
     std::vector<double2> tw(L);
-    for (int k = 0; k < L; ++k) {
-        const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)L;
-        tw[k] = make_double2((double)cosl(a), (double)sinl(a));
-    }
+    std::vector<long double> re(L), im(L);
+    fx_host_roots(L, re.data(), im.data());
+    for (int k = 0; k < L; ++k) tw[k] = make_double2((double)re[k], (double)im[k]);
     int rc = lss_check_cuda(c, cudaMemcpyAsync(c->tw, tw.data(), L * sizeof(double2), cudaMemcpyHostToDevice, s),
                             "twiddles");
     if (rc) return rc;

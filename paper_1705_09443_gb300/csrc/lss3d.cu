@@ -1173,10 +1173,9 @@ int build_kernel3(lss_ctx* c, cudaStream_t s) {
     Ctx3* d = c->d3;
     const int L = c->L, lg = c->lgL;
     std::vector<double2> tw(L);
-    for (int k = 0; k < L; ++k) {
-        const long double a = -2.0L * 3.14159265358979323846264338327950288L * (long double)k / (long double)L;
-        tw[k] = make_double2((double)cosl(a), (double)sinl(a));
-    }
+    std::vector<long double> re(L), im(L);
+    fx_host_roots(L, re.data(), im.data());
+    for (int k = 0; k < L; ++k) tw[k] = make_double2((double)re[k], (double)im[k]);
     int rc = lss_check_cuda(c, cudaMemcpyAsync(c->tw, tw.data(), L * sizeof(double2), cudaMemcpyHostToDevice, s),
                             "twiddles");
     if (rc) return rc;
@@ -1189,6 +1188,7 @@ int build_kernel3(lss_ctx* c, cudaStream_t s) {
     const int nt = line_threads3(L);
     const size_t sh = 2 * (size_t)L * sizeof(double2);
     const int C = col_group3(L);
+    const bool fx = lss_fx_supported(lg);   // the digits take khat's place
     {
         ProfScope ps(c, s, LSS_PROF_SETUP, 4);
         k3_table_circ<<<4 * c->num_sms, 256, 0, s>>>(kc, c->n, L, c->omega, c->h, make_double2(k0.real(), k0.imag()));
@@ -1200,20 +1200,18 @@ int build_kernel3(lss_ctx* c, cudaStream_t s) {
         // along x1, stored transposed and scaled
         const double scale = c->omega * c->omega / ((double)L * L * L);
         mv3_cols<COL_KHAT><<<dim3((unsigned)((long long)L * L / C), 1, 1), C * nt, 2 * (size_t)C * L * sizeof(double2),
-                             s>>>(kc, d->khat, nullptr, c->tw, 1, L, L, (long long)L * L, L, lg, C, scale);
+                             s>>>(kc, fx ? tmp : d->khat, nullptr, c->tw, 1, L, L, (long long)L * L, L, lg, C, scale);
     }
     rc = lss_check_cuda(c, cudaGetLastError(), "3D kernel table");
+    if (!rc && fx) {
+        c->fx_khat = d->khat;
+        d->khat = nullptr;
+        rc = lss_fx_tables(c, tmp, s);
+    }
     cudaError_t e = cudaStreamSynchronize(s);
     cudaFree(kc);
     cudaFree(tmp);
     if (!rc) rc = lss_check_cuda(c, e, "3D kernel table");
-    if (!rc && lss_fx_supported(lg)) {
-        rc = lss_fx_tables(c, d->khat, s);
-        if (!rc) {
-            cudaFree(d->khat);
-            d->khat = nullptr;
-        }
-    }
     return rc;
 }
 

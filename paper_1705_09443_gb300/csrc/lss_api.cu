@@ -37,7 +37,7 @@ void free_ctx(lss_ctx* c) {
     for (auto e : c->iter_ev)
         if (e) cudaEventDestroy(e);
     if (c->host_flags) cudaFreeHost(c->host_flags);
-    void* ptrs[] = {c->m, c->khatT, c->tw, c->fx_tw, c->fx_khat, c->fx_ek, c->gam_phys, c->gam_aux, c->gam_aux_r, c->coef64,
+    void* ptrs[] = {c->m, c->khatT, c->tw, c->fx_tw, c->fx_khat, c->gam_phys, c->gam_aux, c->gam_aux_r, c->coef64,
                     c->coef == c->coef64 ? nullptr : c->coef, c->fac, c->cr_work, c->iface, c->iface_t, c->d_slabs,
                     c->d_err, c->d_bar, c->mv_buf, c->f_buf, c->side_buf, c->z_buf, c->kr_buf, c->red_buf,
                     c->io_buf, c->dir_buf, c->gr_buf, c->ifx_buf, c->ifp_buf, c->gm_buf, c->hz_buf, c->seg_buf,

@@ -136,7 +136,8 @@ struct lss_ctx {
     // digits, kernel transform as digits in storage order and its exponent per line
     void* fx_tw = nullptr;
     void* fx_khat = nullptr;
-    int* fx_ek = nullptr;
+    int* fx_ek = nullptr;         // (part of the fx_tw allocation)
+    std::vector<int> fx_host;     // the digits on the host: the upload may read them after its call
     double2* gam_phys = nullptr;  // (2b+1)^2 x 9 PML stencils (row coefficients)
     double2* gam_aux = nullptr;   // n_samples x b_aux x (2b+1) x 9
     double2* gam_aux_r = nullptr; // the same for the auxiliary PML right of D_i (two fronts)
@@ -275,10 +276,10 @@ enum MvIn { MV_IN_MU = 0, MV_IN_U = 1, MV_IN_PLANEWAVE = 2, MV_IN_RAW = 3 };
 enum MvOut { MV_OUT_A = 0, MV_OUT_AT = 1, MV_OUT_NEG = 2 };
 int lss_matvec(lss_ctx* c, const double2* x, double2* y, int R, int in_mode, int out_mode,
                const double* dirs_dev, double2* uI, cudaStream_t s);
-int lss_fft_kernel_table(lss_ctx* c, const double2* kc, cudaStream_t s);  // kc: L x L -> khatT
+int lss_fft_kernel_table(lss_ctx* c, double2* kc, cudaStream_t s);  // kc: L x L (overwritten) -> khatT or fx_khat
 int lss_fft_configure(lss_ctx* c);
 // the context's fixed-point tables from its kernel transform khat (2D: transposed L x L, 3D: [k2][k3][k1])
-int lss_fx_tables(lss_ctx* c, const double2* khat, cudaStream_t s);
+int lss_fx_tables(lss_ctx* c, const double2* khat, cudaStream_t s);   // digits into c->fx_khat
 std::vector<int> lss_fft_col_candidates(const lss_ctx* c);   // admissible column groups (autotuner)
 // slab.cu: at least n - 1 auxiliary streams (with events) and the fork event
 int lss_ensure_aux(lss_ctx* c, size_t n);
