@@ -33,13 +33,16 @@
  *    then describes the failure.  A failed call leaves the context usable
  *    unless the code is LSS_ERR_CUDA.
  *
- * Environment switches (read at each call; each selects between two exact
- * implementations of the same operation, for comparison and testing):
+ * Environment switches (read at each call, LSS_SOLVE_NR by lss_setup; each
+ * selects between two exact implementations of the same operation, for
+ * comparison and testing):
  *  - LSS_SLAB_SOLVE=cr: 2D slab solves always by the block cyclic reduction
  *    (default: in mixed precision the 16-wide slabs of solves with R >= 16 by
  *    the block LU).
  *  - LSS_BATCH_THREADS=1: a batch context solves each instance on its own
  *    host thread (default: one lockstep Krylov driver for all instances).
+ *  - LSS_SOLVE_NR=2: two right-hand sides per cluster in the cyclic reduction
+ *    of 16-wide slabs (default: four in mixed precision, one in double).
  *  - LSS_TC_UPDATE=0: the 3D mixed factorization's rank updates on CUDA
  *    cores (default: 3xTF32 tcgen05 tensor cores).
  */
@@ -340,7 +343,8 @@ int lss_set_graphs(lss_ctx *c, int enable);
  * blocks the host.  On a batch: every instance.  The paper has no
  * counterpart (launch configuration only).
  *   chosen  host, 7 ints (may be NULL): column group, -1, 0, recurrence
- *           stages, 0, 0, 1 (the constants: the slab solves' automatic choice)
+ *           stages, 0, 0 (the constants: the slab solves' automatic choice),
+ *           right-hand sides per cluster in the slab solves of 16-wide slabs
  */
 int lss_autotune(lss_ctx *c, int R, int *chosen, void *stream);
 

@@ -546,10 +546,8 @@ int launch(lss_ctx* c, CrcArgs A, int nsl, cudaStream_t s) {
 
 template <typename T, int MODE, bool TR>
 int dispatch(lss_ctx* c, const CrcArgs& A, int nsl, int ldw, cudaStream_t s) {
-    // Single precision is bound by the factor stream and by latency: four
-    // right-hand sides share every factor entry (n = 512, 12: 7.0 against 12.3 ms
-    // of pass A per solve).  Double precision is bound by the FP64 pipe: one per
-    // cluster leaves more warps to fill it (n = 256, 8: 1.53 against 2.16 ms).
+    if constexpr (!TR)
+        if (ldw == 16 && lss_cr_cluster_rhs(c, A.R) == 2) return launch<T, MODE, TR, 16, 2>(c, A, nsl, s);
     if constexpr (sizeof(T) == 4)
         if (A.R > 1 && c->n_tot <= 1400)   // (their rows of a 32-wide slab fit 8 CTAs)
             return ldw == 16 ? launch<T, MODE, TR, 16, 4>(c, A, nsl, s) : launch<T, MODE, TR, 32, 4>(c, A, nsl, s);
@@ -557,6 +555,15 @@ int dispatch(lss_ctx* c, const CrcArgs& A, int nsl, int ldw, cudaStream_t s) {
 }
 
 }  // namespace
+
+// Single precision is bound by the factor stream and by latency: four
+// right-hand sides share every factor entry (n = 512, 12: 7.0 against 12.3 ms
+// of pass A per solve).  Double precision is bound by the FP64 pipe: one per
+// cluster leaves more warps to fill it (n = 256, 8: 1.53 against 2.16 ms with four).
+int lss_cr_cluster_rhs(const lss_ctx* c, int R) {
+    if (R > 1 && c->tune.solve_nr == 2) return 2;
+    return c->prec == LSS_MIXED && R > 1 && c->n_tot <= 1400 ? 4 : 1;
+}
 
 int lss_cr_cluster(lss_ctx* c, int mode, bool transpose, CrcArgs A, int s0, int nsl, int ldw, cudaStream_t s) {
     A.slabs = c->d_slabs;

@@ -29,3 +29,6 @@ struct CrcArgs {
 // One pass over the slabs [s0, s0 + nsl) of block width ldw (16 or 32);
 // LSS_ERR_UNSUPPORTED when a slab's rows do not fit a cluster's shared memory.
 int lss_cr_cluster(lss_ctx* c, int mode, bool transpose, CrcArgs A, int s0, int nsl, int ldw, cudaStream_t s);
+
+// Right-hand sides that share a cluster in the forward passes over 16-wide slabs.
+int lss_cr_cluster_rhs(const lss_ctx* c, int R);

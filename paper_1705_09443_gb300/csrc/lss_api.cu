@@ -232,6 +232,8 @@ int lss_setup(lss_ctx** out, const lss_grid* g, double omega, const double* m_de
     c->b_aux = slab->b_aux ? slab->b_aux : pml->b_pml;
     c->n_samples = slab->n_samples ? slab->n_samples : g->n;
     c->fronts = slab->fronts == 2 ? 2 : 1;
+    const char* nr = std::getenv("LSS_SOLVE_NR");
+    if (nr && nr[0] == '2') c->tune.solve_nr = 2;
     c->n_tot = c->n + 2 + 2 * c->b;
     int dev = 0;
     cudaGetDevice(&dev);

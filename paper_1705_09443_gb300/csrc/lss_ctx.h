@@ -184,6 +184,7 @@ struct lss_ctx {
     struct Tune {
         int fft_C = 0;        // columns per CTA of the FFT column pass
         int rec_nb = 0;       // ring stages of the TMA recurrence
+        int solve_nr = 0;     // 2: two right-hand sides per cluster on 16-wide slabs (LSS_SOLVE_NR)
     } tune;
 
     // CUDA graphs of the FGMRES iteration body (preconditioner, operator,

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "cr_cluster.h"
 #include "lss_common.cuh"
 #include "lss_ctx.h"
 
@@ -108,14 +109,15 @@ extern "C" int lss_autotune(lss_ctx* c, int R, int* chosen, void* stream) {
         if (rc) return rc;
     }
     if (chosen) {
-        const lss_ctx::Tune& t = c->inst.empty() ? c->tune : c->inst[0]->tune;
+        const lss_ctx* c0 = c->inst.empty() ? c : c->inst[0];
+        const lss_ctx::Tune& t = c0->tune;
         chosen[0] = t.fft_C;
         chosen[1] = -1;   // the slab solves size themselves (cr_cluster.cu)
         chosen[2] = 0;
         chosen[3] = t.rec_nb;
         chosen[4] = 0;
         chosen[5] = 0;
-        chosen[6] = 1;
+        chosen[6] = lss_cr_cluster_rhs(c0, R);
     }
     return LSS_OK;
 }
