@@ -336,10 +336,11 @@ int lss_set_graphs(lss_ctx *c, int enable);
 /*
  * lss_autotune - pick launch parameters for R right-hand sides by timing this
  * context's own operations (CUDA events, a few runs per candidate): the FFT
- * column group of the LS operator and the recurrence's ring depth (the slab
- * solves size themselves).  2D grids only (LSS_ERR_UNSUPPORTED on a 3D context).  None of them changes any result (same arithmetic, same order),
- * so later solves agree bit for bit with untuned ones; only their speed
- * changes.  Requires a factored context; allocates and frees two vectors;
+ * column group of the LS operator (fixed for the fixed-point line lengths, n
+ * from 17 to 1024, and then only reported) and the recurrence's ring depth (the
+ * slab solves size themselves).  2D grids only (LSS_ERR_UNSUPPORTED on a 3D
+ * context).  None of them changes any result (same arithmetic, same order), so
+ * later solves agree bit for bit with untuned ones; only their speed changes.  Requires a factored context; allocates and frees two vectors;
  * blocks the host.  On a batch: every instance.  The paper has no
  * counterpart (launch configuration only).
  *   chosen  host, 7 ints (may be NULL): column group, -1, 0, recurrence

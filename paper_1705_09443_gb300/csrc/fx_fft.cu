@@ -338,7 +338,10 @@ cudaError_t launch_plan(int mode, int E, const FxArgs& A, int R, cudaStream_t s)
 
 bool lss_fx_supported(int lg) { return lg >= kFxMinLg && lg <= kFxMaxLg; }
 
-int lss_fx_lines(int lg) { return lg <= 10 ? FxPlan<10, 8>::C : FxPlan<11, 8>::C; }
+int lss_fx_lines(int lg) {
+    static_assert(FxPlan<6, 8>::C == FxPlan<9, 8>::C && FxPlan<10, 8>::C == FxPlan<11, 8>::C, "lines per CTA");
+    return lg <= 9 ? FxPlan<9, 8>::C : FxPlan<11, 8>::C;
+}
 
 // Eight entries per thread unless that leaves fewer than 256 threads per SM in
 // the widest pass, then four (n = 64: 22.5 against 30.7 us per application,

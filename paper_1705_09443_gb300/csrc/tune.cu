@@ -59,11 +59,15 @@ int tune_one(lss_ctx* c, int R, cudaStream_t s) {
     Timer t;
     const std::string err0 = c->err;
     const lss_ctx::Tune keep = c->tune;
-    // FFT column group: the LS operator alone
-    {
+    // FFT column group: the LS operator alone (nothing to time where it has one,
+    // as the fixed-point line lengths do)
+    const std::vector<int> groups = lss_fft_col_candidates(c);
+    if (groups.size() == 1) {
+        c->tune.fft_C = groups[0];
+    } else {
         float best = -1;
         int pick = 0;
-        for (int C : lss_fft_col_candidates(c)) {
+        for (int C : groups) {
             c->tune.fft_C = C;
             const float ms = time_ms(t, s, 5, [&] { return lss_matvec(c, x, y, R, MV_IN_MU, MV_OUT_A, nullptr, nullptr, s); });
             if (ms > 0 && (best < 0 || ms < best)) { best = ms; pick = C; }

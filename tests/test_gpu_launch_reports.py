@@ -28,3 +28,9 @@ def test_right_hand_sides_per_cluster(precision, auto, monkeypatch):
     assert s.autotune(1)["solve_rhs_per_cta"] == t.autotune(1)["solve_rhs_per_cta"] == 1
     x = torch.randn((5, 24, 24), dtype=torch.complex128, device="cuda")
     assert torch.equal(s.apply_P(x), t.apply_P(x))
+
+
+@pytest.mark.parametrize("n,lines", [(17, 4), (100, 4), (256, 4), (257, 2), (700, 2)])
+def test_lines_per_cta_of_the_operator(n, lines):
+    """Padded lengths up to 512 have four lines per CTA, above two."""
+    assert make(n, 1).autotune(1)["fft_col_group"] == lines
