@@ -255,6 +255,15 @@ def leg_fronts(w):
     return 2 if w.dim == 2 else 1
 
 
+def slab_solver(dim, R, prec, recursive=False):
+    """How a leg's slabs are solved (the block LU serves mixed precision only)."""
+    if dim == 3:
+        return "recursive (inner sweep along x2)" if recursive else "block elimination of the whole slab along x2"
+    if R >= 16 and prec:
+        return "block LU on 16-wide slabs, cyclic reduction on the others"
+    return "block cyclic reduction"
+
+
 def make_solver(w, m_dev, prec, dev, fronts=None, recursive=None):
     from paper_1705_09443_gb300 import LSSolver
     return LSSolver(w.n, w.omega, m_dev, b_pml=w.b_pml, b_slab=w.b_slab, precision=prec,
@@ -404,10 +413,7 @@ def run_leg(args, dev, world, flush, wname, prec, steps, warmup, recursive=False
     prof_ms, prof_n = profile_pass(s, step, 1)
     flat = [x for st in stats for x in st]
     out = {"workload": wname, "precision": "mixed" if prec else "fp64", "R": R, "fronts": leg_fronts(w),
-           "slab_solver": ("recursive (inner sweep along x2)" if recursive else
-                           "block elimination of the whole slab along x2" if w.dim == 3 else
-                           "block LU on 16-wide slabs, cyclic reduction on the others" if R >= 16 else
-                           "block cyclic reduction"),
+           "slab_solver": slab_solver(w.dim, R, prec, recursive),
            "value": R * steps * world / (tot / 1e3), "unit": "solves/s", "ms_per_step": tot / steps,
            "solve_only": {"value": R * steps * world / (sum(ts_s) / 1e3), "ms_per_solve_call": sum(ts_s) / steps},
            "setup_factor_ms": float(ts_f[0]), "iters": float(np.mean([x["iters"] for x in flat])),
