@@ -480,12 +480,12 @@ __device__ __forceinline__ void warp_pivot(float& v, int& row) {
     row = (int)__reduce_min_sync(0xffffffffu, u == m ? (unsigned)row : 0x7fffffffu);
     v = __uint_as_float(m);
 }
-__device__ __forceinline__ void warp_pivot(double& v, int& row) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, row, o);
-        if (ov > v || (ov == v && oi < row)) { v = ov; row = oi; }
-    }
+__device__ __forceinline__ void warp_pivot(double& v, int& row) {   // (FP64 compares would take the FP64 pipe)
+    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+    const unsigned mh = __reduce_max_sync(0xffffffffu, h);
+    const unsigned ml = __reduce_max_sync(0xffffffffu, h == mh ? l : 0u);
+    row = (int)__reduce_min_sync(0xffffffffu, h == mh && l == ml ? (unsigned)row : 0x7fffffffu);
+    v = __hiloint2double((int)mh, (int)ml);
 }
 
 // Gauss-Jordan elimination of the panel columns J = [j0, j0+nbp) of W (one
@@ -505,6 +505,9 @@ __device__ __forceinline__ void warp_pivot(double& v, int& row) {
 // M = 984 .. 1476, 16 columns, FP32: 30 us (67 with the panel of a slab in one
 // CTA's shared memory, 52 in one CTA's registers, which spill at three rows per
 // thread; unrolled over the pivots 80, bound by the instruction fetch).
+// FP64 is bound by its pipe, so only rows that exist reach it (M = 64 .. 100, whole
+// factorization of the recursive approach at n = 20: 35.7 ms; 50.5 with every
+// thread's update and comparisons in FP64, 40.4 with one CTA's shared memory).
 constexpr int kPanelThreads = 448, kPanelCtas = 4;
 static_assert(kMaxBlock3 <= kPanelThreads * kPanelCtas, "rows of the widest pivot block");
 
@@ -608,10 +611,12 @@ __global__ void __launch_bounds__(kPanelThreads) f3_panel(const Slab3* __restric
 #pragma unroll
             for (int q = 0; q < NB; ++q) x[q] = s_old[par][q];
         }
-        const C l = czero<C>() - x[0] * d;
+        if (sizeof(R) == 4 || r < M) {   // warps without rows leave the FP64 pipe to the others
+            const C l = czero<C>() - x[0] * d;
 #pragma unroll
-        for (int q = 1; q < NB; ++q) x[q - 1] = cfma(l, pn[q], x[q]);
-        x[NB - 1] = l;
+            for (int q = 1; q < NB; ++q) x[q - 1] = cfma(l, pn[q], x[q]);
+            x[NB - 1] = l;
+        }
     }
     __syncthreads();
     if (r < M)
