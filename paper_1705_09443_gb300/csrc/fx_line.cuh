@@ -1,7 +1,7 @@
 // Line FFTs of the LS operator in 64-bit fixed point.
 //
-// This GPU issues 1.6 FP64 operations per clock and SM but about 24 32 x 32 ->
-// 64-bit integer multiply-adds and 110 integer adds (measured): an FFT in
+// This GPU issues 2 FP64 multiply-adds per clock and SM but 14 to 22 32 x 32 ->
+// 64-bit integer ones and 122 32-bit additions (probe, 32 warps per SM): an FFT in
 // 64-bit integers takes a fraction of the FP64 pipe's time, which bounded the
 // operator (n = 512, 64 right-hand sides: 13.4 -> 3.24 ms; 3D n = 64: 365 ->
 // 136 us).  A line is held as integers with one exponent, v * 2^E, scaled so

@@ -506,7 +506,7 @@ __device__ __forceinline__ void warp_pivot(double& v, int& row) {   // (FP64 com
 // CTA's shared memory, 52 in one CTA's registers, which spill at three rows per
 // thread; unrolled over the pivots 80, bound by the instruction fetch).
 // FP64 is bound by its pipe, so only rows that exist reach it (M = 64 .. 100, whole
-// factorization of the recursive approach at n = 20: 35.7 ms; 50.5 with every
+// factorization of the recursive approach at n = 20: 35.4 ms; 50.5 with every
 // thread's update and comparisons in FP64, 40.4 with one CTA's shared memory).
 constexpr int kPanelThreads = 448, kPanelCtas = 4;
 static_assert(kMaxBlock3 <= kPanelThreads * kPanelCtas, "rows of the widest pivot block");

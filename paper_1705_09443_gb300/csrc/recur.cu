@@ -7,15 +7,15 @@
 // chain passes, with no barrier inside.  A chain step is one product of an
 // n_tot x n_tot map with the n_tot x R vectors (two with two fronts), a grid
 // barrier closes it.  What bounds a step is latency and, in FP64, the FP64
-// pipe (1.6 operations per clock and SM), so a step has to reach every SM: a
+// pipe (2 multiply-adds per clock and SM), so a step has to reach every SM: a
 // task is only TRC = 8, 4, 2 or 1 rows of CW columns, its length-n_tot sums
 // split over the 16 warps of a CTA (lanes along the columns, so vector rows
 // are read coalesced and map entries are broadcast from shared memory, a
 // partial sum per warp added up at the end).  A CTA's next map rows do not
 // depend on the chain and are copied by cp.async before the barrier.
-// FP64, n = 256, 16 right-hand sides, one front: 2.4 ms per sweep against 19.1
-// of 16-column tiles
-// of 32 rows, which left 18 CTAs per step; FP32, n = 512, 64 right-hand
+// FP64, n = 256, 16 right-hand sides, one front: 2.4 ms per sweep (the FP64 pipe
+// 70 % busy) against 19.1 of 16-column tiles of 32 rows, which left 18 CTAs per
+// step; FP32, n = 512, 64 right-hand
 // sides, two fronts: 2.05 ms against 3.35.
 #include <algorithm>
 #include <mutex>

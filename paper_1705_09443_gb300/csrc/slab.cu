@@ -1964,10 +1964,12 @@ int prepare_chunk_tables(lss_ctx* c, cudaStream_t s) {
 }
 
 // The block LU's right-hand sides share a chain of 2 n_tot block rows per CTA,
-// which pays where the arithmetic is cheap: in double precision 65 x 1 CTAs
-// (n = 256, 16 right-hand sides) took 14 ms per pass, bound by the FP64 pipe
-// of 65 SMs, the cluster solves (cr_cluster.cu) 2.9.  In single precision at
-// n = 512 with 64 it takes 4.1 ms per pass where they take 5.5.
+// which pays where the arithmetic is cheap.  In double precision it is bound by
+// the FP64 pipe, by that of 65 SMs with 65 x 1 CTAs (n = 256, 16 right-hand
+// sides: 14 ms per pass against 2.9 of the cluster solves, cr_cluster.cu) and
+// still where its CTAs cover the GPU (P, two fronts, block LU / clusters: n = 512
+// with 32 99 / 68 ms, with 64 193 / 134; one front with 64 170 / 134).  In
+// single precision at n = 512 with 64 it takes 2.4 ms per pass where they take 5.5.
 // LSS_SLAB_SOLVE=cr: cyclic reduction for every run.
 bool thomas_enabled(const lss_ctx* c) {
     if (c->prec == LSS_FP64) return false;
