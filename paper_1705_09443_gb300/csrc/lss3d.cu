@@ -502,11 +502,11 @@ __device__ __forceinline__ void warp_pivot(double& v, int& row) {   // (FP64 com
 // one register per pivot (the pivot column is always register 0), which keeps
 // the loop rolled.  Rows reach the registers through a swizzled tile, so that W
 // is read and written in whole segments.
-// M = 984 .. 1476, 16 columns, FP32: 30 us (67 with the panel of a slab in one
+// M = 984 .. 1476, 16 columns, FP32: 32 us (67 with the panel of a slab in one
 // CTA's shared memory, 52 in one CTA's registers, which spill at three rows per
 // thread; unrolled over the pivots 80, bound by the instruction fetch).
 // FP64 is bound by its pipe, so only rows that exist reach it (M = 64 .. 100, whole
-// factorization of the recursive approach at n = 20: 35.4 ms; 50.5 with every
+// factorization of the recursive approach at n = 20: 37.3 ms; 50.5 with every
 // thread's update and comparisons in FP64, 40.4 with one CTA's shared memory).
 constexpr int kPanelThreads = 448, kPanelCtas = 4;
 static_assert(kMaxBlock3 <= kPanelThreads * kPanelCtas, "rows of the widest pivot block");
@@ -602,7 +602,10 @@ __global__ void __launch_bounds__(kPanelThreads) f3_panel(const Slab3* __restric
             }
         }
         // new row j = d times the pivot row; every other row (row pr taking the
-        // old row j's values) eliminated: x_q -= (x_jj d) p_q, x_jj = -x_jj d
+        // old row j's values) eliminated: x_q -= (x_jj d) p_q, x_jj = -x_jj d.
+        // Product first, then one rounding at the size of x_q: multiply-adds into
+        // x_q round there twice, and put P in mixed precision 7 to 11 % further
+        // from FP64 (n = 6 to 32).
         if (r == j) {   // 0 + d p_q
 #pragma unroll
             for (int q = 1; q < NB; ++q) x[q] = czero<C>();
@@ -614,7 +617,7 @@ __global__ void __launch_bounds__(kPanelThreads) f3_panel(const Slab3* __restric
         if (sizeof(R) == 4 || r < M) {   // warps without rows leave the FP64 pipe to the others
             const C l = czero<C>() - x[0] * d;
 #pragma unroll
-            for (int q = 1; q < NB; ++q) x[q - 1] = cfma(l, pn[q], x[q]);
+            for (int q = 1; q < NB; ++q) x[q - 1] = x[q] + l * pn[q];
             x[NB - 1] = l;
         }
     }
