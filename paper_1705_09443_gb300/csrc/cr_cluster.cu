@@ -10,7 +10,8 @@
 // blocks and 8 of the inverse per lane, coalesced), those of a level's first
 // task before the barrier, so that the factor latency overlaps it.  A 16-wide
 // row is a warp's task (a half warp per block), a 32-wide row that of four
-// warps (block x half of the columns, partial sums through shared memory).
+// warps (block x half of the columns, partial sums through shared memory).  A CTA
+// has 256 threads for 16-wide slabs, 512 or 256 for 32-wide ones (launch).
 //
 // Forward operator, level by level:
 //   P0     y_o = D_o^{-1} b_o on the odd rows
@@ -32,9 +33,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-template <int G>
-constexpr int crc_threads() { return G == 16 ? 256 : 512; }
-
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
@@ -45,12 +43,15 @@ __device__ __forceinline__ C shfl_xor_c(C v, int o) {
     return v;
 }
 
-template <typename T, int MODE, bool TR, int G, int NR>
+template <typename T, int MODE, bool TR, int G, int NR, int NT>
 struct Crc {
     using C = cx<T>;
-    static constexpr int NT = crc_threads<G>();
     static constexpr int TW = G == 16 ? 1 : 4;                 // warps per task
     static constexpr int kTeams = NT / 32 / TW;
+    // Columns beyond the layers of a 32-wide slab are zero.  FP64 is bound by its
+    // pipe and neither reads nor multiplies them (20 layers, n = 64, 16 right-hand
+    // sides: P 1.33 -> 1.16 ms); in FP32 the test takes longer than it saves.
+    static constexpr bool kSkip = G == 32 && sizeof(T) == 8;
     static constexpr int XS = 18;                              // staged entries of one vector (16, padded for the banks)
     static constexpr int kStage = (G == 16 ? 2 : 1) * NR * XS; // per warp
     static constexpr int kPart = G == 16 ? 0 : 2 * 4 * NR * 32;   // per team: partial sums, two buffers
@@ -66,6 +67,7 @@ struct Crc {
     int K, P, rank, lo, hi;   // own rows [lo, hi)
     int lane, p, sub, team;   // p: layer; sub: which part of a task this half warp / warp has
     int nc;                   // right-hand sides
+    int kp, ki;               // columns within the slab's layers of this lane's part of a pair, of an inverse
     int buf = 0;
 
     C m[16], d[8];
@@ -85,6 +87,8 @@ struct Crc {
         rank = (int)cl.block_rank();
         lo = min(K, rank * P);
         hi = min(K, lo + P);
+        kp = max(0, min(16, sd.w - ca()));
+        ki = max(0, min(8, sd.w - sub * 8));
     }
     // column c of the block row at position k, in whichever CTA owns it
     __device__ const C* row(int k, int c) const {
@@ -99,7 +103,7 @@ struct Crc {
     __device__ void load_inv(long long block) {
         const C* M = F + block * (G * G);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) d[u] = ent(M, p, sub * 8 + u);
+        for (int u = 0; u < 8; ++u) d[u] = !kSkip || u < ki ? ent(M, p, sub * 8 + u) : czero<C>();
     }
     // the part of a pair of blocks that this lane multiplies: the left
     // neighbour's block or the right one's, columns ca .. ca + 15
@@ -109,7 +113,7 @@ struct Crc {
         const bool has = side() ? hr : hl;
         const C* M = side() ? right : left;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) m[u] = has ? ent(M, p, ca() + u) : czero<C>();
+        for (int u = 0; u < 16; ++u) m[u] = has && (!kSkip || u < kp) ? ent(M, p, ca() + u) : czero<C>();
     }
     // acc[c] = this lane's part of  (left) x_{kl} + (right) x_{kr}
     __device__ void pair(int kl, int kr, bool hl, bool hr, C (&acc)[NR]) {
@@ -130,6 +134,7 @@ struct Crc {
                 C s1 = czero<C>();
 #pragma unroll
                 for (int u = 0; u < 16; u += 2) {
+                    if (kSkip && u >= kp) break;
                     acc[c] = cfma(m[u], s[c * XS + u], acc[c]);
                     s1 = cfma(m[u + 1], s[c * XS + u + 1], s1);
                 }
@@ -159,6 +164,7 @@ struct Crc {
                 C s1 = czero<C>();
 #pragma unroll
                 for (int u = 0; u < 8; u += 2) {
+                    if (kSkip && u >= ki) break;
                     acc[c] = cfma(d[u], s[c * XS + u], acc[c]);
                     s1 = cfma(d[u + 1], s[c * XS + u + 1], s1);
                 }
@@ -468,14 +474,14 @@ struct Crc {
     }
 };
 
-template <typename T, int MODE, bool TR, int G, int NR>
-__global__ void __launch_bounds__(crc_threads<G>(), G == 16 ? 2 : 1) cr_cluster_kernel(const __grid_constant__ CrcArgs A) {
+template <typename T, int MODE, bool TR, int G, int NR, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) cr_cluster_kernel(const __grid_constant__ CrcArgs A) {
     extern __shared__ __align__(128) unsigned char crc_smem[];
     const int i = A.slab0 + blockIdx.y;
     __shared__ SlabDev sd;
     if (threadIdx.x == 0) sd = A.slabs[i];
     __syncthreads();
-    Crc<T, MODE, TR, G, NR> S(A, sd, reinterpret_cast<cx<T>*>(crc_smem));
+    Crc<T, MODE, TR, G, NR, NT> S(A, sd, reinterpret_cast<cx<T>*>(crc_smem));
     const int r0 = (int)(blockIdx.x / S.cl.num_blocks()) * NR;
     S.nc = min(NR, A.R - r0);
     S.solve(i, r0);
@@ -483,13 +489,24 @@ __global__ void __launch_bounds__(crc_threads<G>(), G == 16 ? 2 : 1) cr_cluster_
 
 constexpr size_t kCrcSmem = size_t(220) * 1024;
 
-template <typename T, int MODE, bool TR, int G, int NR>
+// Clusters of a pass's slabs of one width.
+int crc_clusters(const lss_ctx* c, int ldw, int R, int nr) {
+    int total = 0;   // (its runs share the SMs)
+    for (const SlabDev& q : c->slabs) total += q.ldw == ldw;
+    return total * ((R + nr - 1) / nr);
+}
+// Clusters of cl CTAs that the GPU holds at once, a CTA per SM: a cluster lies in
+// one GPC (18 to 20 SMs), so 16 clusters of 8 or 36 of 4 fill it.
+bool crc_one_wave(const lss_ctx* c, long long clusters, int cl) {
+    return clusters * cl <= (cl == 8 ? c->num_sms * 6 / 7 : c->num_sms * 19 / 20);
+}
+
+template <typename T, int MODE, bool TR, int G, int NR, int NT>
 int launch(lss_ctx* c, CrcArgs A, int nsl, cudaStream_t s) {
-    int total = 0;   // slabs of this width in the whole pass (its runs share the SMs)
-    for (const SlabDev& q : c->slabs) total += q.ldw == G;
-    using S = Crc<T, MODE, TR, G, NR>;
-    auto kern = cr_cluster_kernel<T, MODE, TR, G, NR>;
+    using S = Crc<T, MODE, TR, G, NR, NT>;
+    auto kern = cr_cluster_kernel<T, MODE, TR, G, NR, NT>;
     const int K = A.n_tot, groups = (A.R + NR - 1) / NR;
+    const long long N = crc_clusters(c, G, A.R, NR);
     auto smem = [&](int P) { return sizeof(cx<T>) * ((size_t)S::kFixed + (size_t)P * NR * G); };
     // Cluster size.  More CTAs per slab shorten the chain of the low levels but
     // make the barriers of the high ones dearer, and once the pass fills the
@@ -498,23 +515,33 @@ int launch(lss_ctx* c, CrcArgs A, int nsl, cudaStream_t s) {
     // n = 181, 1 680 / 410 / 400, n = 256, 8 3170 / 3110 / 3350; mixed n = 256,
     // 1 (two fronts) 320 / 200 / 245, n = 512, 1 600 / 630 / 410 (few CTAs of
     // many rows lack loads in flight: at least two CTAs where 128 rows remain).
-    // 32-wide slabs are few and four times the work, so theirs is the longest
-    // chain: 8 CTAs (FP64 n = 256, 1: 1000 us, with 4 1070 and with 2 1490;
-    // clusters of 16 take longer in mixed precision, n = 256: 360 us against 200).
+    // A 32-wide slab is four times the work.  Where they are few, theirs is the
+    // longest chain: 8 CTAs as long as all clusters run at once, then 4 (FP64
+    // n = 256, 1: 1000 us, with 4 1070 and with 2 1490; clusters of 16 take longer
+    // in mixed precision, n = 256: 360 us against 200).  More clusters than that
+    // come in waves, and two CTAs of 256 threads share an SM to overlap their
+    // barriers, in clusters of 4, of 2 once the SMs are full without (P, ms, 512
+    // threads with 1 / 2 / 4 / 8 CTAs | 256 threads: FP64, all slabs 20 layers wide,
+    // n = 64, 6 right-hand sides 1.01 / 0.65 / 0.71 / 0.88 | 1.12 / 0.71 / 0.62 / 0.69,
+    // 40: 3.12 / 2.92 / 3.36 / 4.92 | 3.11 / 2.77 / 2.87 / 3.44, n = 256, 10:
+    // 8.1 / 7.2 / 7.7 / 9.9 | 7.0 / 7.0 / 6.5 / 7.3; mixed, n = 64, 3:
+    // 0.36 / 0.24 / 0.18 / 0.15, n = 100, 40: 0.86 / 0.90 / 0.97 / 1.17 | 0.83 / 0.83 / 0.84 / 0.93).
     // Beside a block LU of the other slabs the SMs are not theirs alone: 4 CTAs
     // of more than 32 rows each (P, mixed, ms, with 8 / 4 / 2 CTAs: n = 64, 64
     // right-hand sides 1.47 / 1.47 / 1.39, n = 128, 64 3.31 / 3.08 / 3.07 and 96
     // 1.36 / 1.30 / 1.43, n = 256, 32 2.13 / 1.95 / 1.95).
     int cl = 1;
     if (G == 16) {
-        while (cl < 4 && K > 4 * cl && ((long long)total * groups * cl < c->num_sms * 3 / 4 || K / (2 * cl) >= 128))
+        while (cl < 4 && K > 4 * cl && (N * cl < c->num_sms * 3 / 4 || K / (2 * cl) >= 128))
             cl *= 2;
+    } else if (A.beside) {
+        while (cl < 4 && K > 64 * cl && N * cl < c->num_sms) cl *= 2;
     } else {
-        const int most = A.beside ? 4 : 8, rows = A.beside ? 64 : 4;
-        while (cl < most && K > rows * cl && (long long)total * groups * cl < c->num_sms) cl *= 2;
+        cl = NT == 256 ? (N <= 2 * c->num_sms ? 4 : 2) : crc_one_wave(c, N, 8) ? 8 : 4;
+        while (cl > 1 && K <= 2 * cl) cl /= 2;
     }
-    // two CTAs per SM for the 16-wide slabs; past 8 CTAs only where the rows fit no other way
-    while (cl < 8 && smem((K + cl - 1) / cl) > (G == 16 ? kCrcSmem / 2 : kCrcSmem)) cl *= 2;
+    // two CTAs of 256 threads per SM; past 8 CTAs only where the rows fit no other way
+    while (cl < 8 && smem((K + cl - 1) / cl) > (NT == 256 ? kCrcSmem / 2 : kCrcSmem)) cl *= 2;
     if (smem((K + cl - 1) / cl) > kCrcSmem) cl = 16;
     A.P = (K + cl - 1) / cl;
     const size_t sh = smem(A.P);
@@ -532,7 +559,7 @@ int launch(lss_ctx* c, CrcArgs A, int nsl, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3(cl * groups, nsl);
-    cfg.blockDim = dim3(S::NT);
+    cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = sh;
     cfg.stream = s;
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -544,14 +571,20 @@ int launch(lss_ctx* c, CrcArgs A, int nsl, cudaStream_t s) {
     return lss_check_cuda(c, cudaLaunchKernelEx(&cfg, kern, A), "slab solve launch");
 }
 
+template <typename T, int MODE, bool TR, int NR>
+int launch_wide(lss_ctx* c, const CrcArgs& A, int nsl, cudaStream_t s) {
+    if (!A.beside && !crc_one_wave(c, crc_clusters(c, 32, A.R, NR), 4)) return launch<T, MODE, TR, 32, NR, 256>(c, A, nsl, s);
+    return launch<T, MODE, TR, 32, NR, 512>(c, A, nsl, s);
+}
+
 template <typename T, int MODE, bool TR>
 int dispatch(lss_ctx* c, const CrcArgs& A, int nsl, int ldw, cudaStream_t s) {
     if constexpr (!TR)
-        if (ldw == 16 && lss_cr_cluster_rhs(c, A.R) == 2) return launch<T, MODE, TR, 16, 2>(c, A, nsl, s);
+        if (ldw == 16 && lss_cr_cluster_rhs(c, A.R) == 2) return launch<T, MODE, TR, 16, 2, 256>(c, A, nsl, s);
     if constexpr (sizeof(T) == 4)
         if (A.R > 1 && c->n_tot <= 1400)   // (their rows of a 32-wide slab fit 8 CTAs)
-            return ldw == 16 ? launch<T, MODE, TR, 16, 4>(c, A, nsl, s) : launch<T, MODE, TR, 32, 4>(c, A, nsl, s);
-    return ldw == 16 ? launch<T, MODE, TR, 16, 1>(c, A, nsl, s) : launch<T, MODE, TR, 32, 1>(c, A, nsl, s);
+            return ldw == 16 ? launch<T, MODE, TR, 16, 4, 256>(c, A, nsl, s) : launch_wide<T, MODE, TR, 4>(c, A, nsl, s);
+    return ldw == 16 ? launch<T, MODE, TR, 16, 1, 256>(c, A, nsl, s) : launch_wide<T, MODE, TR, 1>(c, A, nsl, s);
 }
 
 }  // namespace
